@@ -13,10 +13,7 @@
 
 namespace pfk {
 
-constexpr int kBaseThreads = 128;
-constexpr int kBaseBlocksPerSm = 6;
-constexpr int kBaseStride = kBaseThreads + 1;
-static_assert(kBaseBlocksPerSm <= kMaxBlocksPerSm, "partials are sized for kMaxBlocksPerSm blocks per SM");
+static_assert(kWinBlocksPerSm <= kMaxBlocksPerSm, "partials are sized for kMaxBlocksPerSm blocks per SM");
 
 // A CSR operator (stencil operators take the tiled walk).
 struct CsrView {
@@ -56,77 +53,60 @@ __global__ void __launch_bounds__(kThreads) base_advance(double* __restrict__ x,
 }
 
 // Dots of a vector v with r (<v, r>), of r with itself, and with the stored
-// s_k of the window W_i (transposed through shared memory).  Mode FCG:
-// v = u = B(r_i): convergence test on gamma_i = <u_i, r_i>, then the betas.
-// Mode GCR: v = A u_i: the betas only.
+// s_k of the window W_i (window_dots).  Mode FCG: v = u = B(r_i): convergence
+// test on gamma_i = <u_i, r_i>, then the betas.  Mode GCR: v = A u_i: the betas
+// only.
 enum { kDotsFcg = 0, kDotsGcr = 1 };
 
 template <int NW>
-__global__ void __launch_bounds__(kBaseThreads, kBaseBlocksPerSm) base_window_dots(const double* __restrict__ v,
-                                                                                   const double* __restrict__ r,
-                                                                                   const double* __restrict__ S,
-                                                                                   int64_t N, SolveCtl* ctl,
-                                                                                   double* partials, int mode) {
+__global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) base_window_dots(const double* __restrict__ v,
+                                                                                 const double* __restrict__ r,
+                                                                                 const double* __restrict__ S,
+                                                                                 int64_t N, SolveCtl* ctl,
+                                                                                 double* partials, int mode) {
   if (ctl->status != kRun) return;
   constexpr int ND = NW + 2;
-  constexpr int NWARPS = kBaseThreads / 32;
+  constexpr int NWARPS = kWinThreads / 32;
   __shared__ size_t s_off[NW];
-  __shared__ double s_sk[NW * kBaseStride];
-  __shared__ double s_v[kBaseThreads];
   __shared__ double s_red[NWARPS * ND];
   __shared__ double s_sum[ND];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = ctl->i + 1;
   const int nu = nu_window(i, ctl->mmax, ctl->truncation);
   const int slots = ctl->mmax + 1;
+  const int ng = mode == kDotsFcg ? 2 : 0;   // <v, r> and <r, r> after the window's dots
   if (threadIdx.x < nu) s_off[threadIdx.x] = (size_t)((i - nu + (int)threadIdx.x) % slots) * (size_t)N;
   __syncthreads();
-  double* my = s_sk + threadIdx.x;
-  const double* wv = s_v + warp * 32;
-  const double* lrow = s_sk + lane * kBaseStride + warp * 32;
-  double g0 = 0.0, g1 = 0.0, gw = 0.0;
-  for (int64_t base = (int64_t)blockIdx.x * kBaseThreads; base < N; base += (int64_t)gridDim.x * kBaseThreads) {
-    const int64_t e = base + threadIdx.x;
-    double vv = 0.0;
-    if (e < N) {
-      vv = v[e];
-      const double rv = r[e];
-      g0 = fma(vv, rv, g0);
-      g1 = fma(rv, rv, g1);
-#pragma unroll
-      for (int j = 0; j < NW; ++j)
-        if (j < nu) my[j * kBaseStride] = S[s_off[j] + e];
-    } else {
-#pragma unroll
-      for (int j = 0; j < NW; ++j)
-        if (j < nu) my[j * kBaseStride] = 0.0;
+  double g0 = 0.0, g1 = 0.0, acc[NW];
+  window_dots<NW>(v, S, s_off, nu, N, acc, [&](int64_t e, double ve) {
+    if (ng) {
+      const double re = __ldg(&r[e]);
+      g0 = fma(ve, re, g0);
+      g1 = fma(re, re, g1);
     }
-    s_v[threadIdx.x] = vv;
-    __syncwarp();
-    if (lane < nu) {
-      double c = gw;
-#pragma unroll 8
-      for (int t = 0; t < 32; ++t) c = fma(wv[t], lrow[t], c);
-      gw = c;
-    }
-    __syncwarp();
-  }
+  });
   {
-    const double w0 = warp_sum(g0), w1 = warp_sum(g1);
-    const int nd = nu + 2;
-    if (lane == 0) {
-      s_red[warp * nd + 0] = w0;
-      s_red[warp * nd + 1] = w1;
+    const double tot = warp_sum_transposed<NW>(acc);
+    const int nd = nu + ng;
+    if (lane < nu) s_red[warp * nd + lane] = tot;
+    if (ng) {
+      double g[2] = {g0, g1};
+      const double w = warp_sum_transposed<2>(g);
+      if (lane < 2) s_red[warp * nd + nu + lane] = w;
     }
-    if (lane < nu) s_red[warp * nd + 2 + lane] = gw;
     __syncthreads();
   }
-  if (!combine_block_partials_2l(s_red, nu + 2, partials, ND, &ctl->counter, ctl->gcounter, s_sum)) return;
+  if (!combine_block_partials_2l(s_red, nu + ng, partials, ND, &ctl->counter, ctl->gcounter, s_sum)) return;
+  // beta_{i,k} = -<v, s_k> / eta_k, one division per thread (a serial loop of
+  // nu divisions in one thread took 25-30 us at nu = 30); not used when the
+  // iteration stops here
+  if ((int)threadIdx.x < nu)
+    ctl->beta[threadIdx.x] = -s_sum[threadIdx.x] / ctl->eta_ring[(i - nu + (int)threadIdx.x) % slots];
   if (threadIdx.x != 0) return;
-  const double* c = s_sum + 2;
+  ctl->nw = nu;
   if (mode == kDotsFcg) {
-    // Alg. 2: gamma_i = <u_i, r_i>, convergence, beta_{i,k} = -<u_i, s_k> / eta_k
-    const double gamma = s_sum[0], rr = s_sum[1];
+    // Alg. 2: gamma_i = <u_i, r_i>, convergence
+    const double gamma = s_sum[nu], rr = s_sum[nu + 1];
     ctl->it += 1;
     ctl->gamma = gamma;
     const double rho = cgcr_rho(ctl, gamma, rr);
@@ -135,8 +115,6 @@ __global__ void __launch_bounds__(kBaseThreads, kBaseBlocksPerSm) base_window_do
     if (!isfinite(rho)) { ctl->status = kNonFinite; return; }
     if (rho <= ctl->target) { ctl->status = kConverged; ctl->i = i; return; }
   }
-  for (int jj = 0; jj < nu; ++jj) ctl->beta[jj] = -c[jj] / ctl->eta_ring[(i - nu + jj) % slots];
-  ctl->nw = nu;
 }
 
 // p_i = u + sum_k beta_{i,k} p_k over W_i, into ring slot i.
@@ -163,19 +141,39 @@ __global__ void __launch_bounds__(kThreads, 3) base_maxpy(const double* __restri
   }
 }
 
-// s = A p for p in ring slot `which` (0 = slot 0, 1 = slot i of the current
-// iteration), with the dots <p, r>, <p, s>, <r, s>, <s, s>, <r, r>; the last
-// block runs the mode's scalar step.
+// s = A p for p in ring slot 0 (fills) or slot i of the current iteration,
+// with the dots its scalar step reads: <p, s> (FCG eta), <p, s>, <p, r>,
+// <r, r> (FCG fill) or <s, s>, <r, s>, <r, r> (GCR fill and final); the last
+// block runs the scalar step.  Only these products are formed: with all five
+// dots of <p, r>, <p, s>, <r, s>, <s, s>, <r, r> the FCG walk issued 12 FP64
+// instructions per cell instead of 8.
 enum { kApplyFcgFill = 0, kApplyFcgEta = 1, kApplyGcrFill = 2, kApplyGcrFinal = 3 };
 
-// The scalar step after s = A p and its five dots (last block, one thread).
-__device__ __forceinline__ void base_apply_scalars(SolveCtl* ctl, int i, int slots, int mode, const double* s_sum) {
-  const double pr = s_sum[0], ps = s_sum[1], rs = s_sum[2], ss = s_sum[3], rr = s_sum[4];
-  if (mode == kApplyFcgFill) { cgcr_fill_scalars(ctl, pr, ps, rr); return; }        // gamma_0 = <u_0, r_0>, eta_0 = <p_0, s_0>
-  if (mode == kApplyGcrFill) { cgcr_fill_scalars(ctl, rs, ss, rr); return; }        // gamma_0 = <r_0, s_0>, eta_0 = <s_0, s_0>
-  if (mode == kApplyFcgEta) {
+template <int MODE>
+struct ApplyDots {
+  static constexpr bool fcg = MODE == kApplyFcgFill || MODE == kApplyFcgEta;
+  static constexpr int nd = MODE == kApplyFcgEta ? 1 : 3;
+  static __device__ __forceinline__ void add(double (&acc)[nd], double pv, double sv, double rv) {
+    acc[0] = fma(fcg ? pv : sv, sv, acc[0]);
+    if constexpr (nd == 3) {
+      acc[1] = fma(rv, fcg ? pv : sv, acc[1]);
+      acc[2] = fma(rv, rv, acc[2]);
+    }
+  }
+};
+
+// The scalar step after s = A p and its dots (last block, one thread): q0 =
+// <p, s> or <s, s>, q1 = <p, r> or <r, s>, rr = <r, r>.
+template <int MODE>
+__device__ __forceinline__ void base_apply_scalars(SolveCtl* ctl, int i, int slots, double q0, double q1, double rr) {
+  if (MODE == kApplyFcgFill || MODE == kApplyGcrFill) {
+    // FCG: gamma_0 = <u_0, r_0>, eta_0 = <p_0, s_0>; GCR: gamma_0 = <r_0, s_0>, eta_0 = <s_0, s_0>
+    cgcr_fill_scalars(ctl, q1, q0, rr);
+    return;
+  }
+  if (MODE == kApplyFcgEta) {
     // Alg. 2: eta_i = <p_i, s_i>, alpha_i = gamma_i / eta_i
-    const double eta = ps;
+    const double eta = q0;
     const double al = eta != 0.0 ? ctl->gamma / eta : nan("");
     ctl->i = i;
     ctl->eta = eta;
@@ -191,6 +189,7 @@ __device__ __forceinline__ void base_apply_scalars(SolveCtl* ctl, int i, int slo
   }
   // Alg. 9 (standard reading): gamma_i = <r_i, s_i>, eta_i = <s_i, s_i>; convergence,
   // then alpha_i = gamma_i / eta_i
+  const double ss = q0, rs = q1;
   ctl->it += 1;
   ctl->i = i;
   ctl->gamma = rs;
@@ -208,85 +207,77 @@ __device__ __forceinline__ void base_apply_scalars(SolveCtl* ctl, int i, int slo
 }
 
 // CSR operators: one row per thread.
+template <int MODE>
 __global__ void __launch_bounds__(kThreads) base_apply_dots(CsrView A, double* __restrict__ P,
                                                             double* __restrict__ S, const double* __restrict__ r,
-                                                            int64_t N, SolveCtl* ctl, double* partials, int mode) {
+                                                            int64_t N, SolveCtl* ctl, double* partials) {
   if (ctl->status != kRun) return;
-  const bool fill = (mode == kApplyFcgFill || mode == kApplyGcrFill);
+  using D = ApplyDots<MODE>;
+  const bool fill = (MODE == kApplyFcgFill || MODE == kApplyGcrFill);
   const int i = fill ? 0 : ctl->i + 1;
   const int slots = ctl->mmax + 1;
   const size_t off = (size_t)(i % slots) * (size_t)N;
   const double* p = P + off;
   double* s = S + off;
-  double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  double acc[D::nd] = {};
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N; e += (int64_t)gridDim.x * blockDim.x) {
     const double sv = base_row(A, p, e);
     s[e] = sv;
-    const double pv = p[e], rv = r[e];
-    acc[0] = fma(pv, rv, acc[0]);
-    acc[1] = fma(pv, sv, acc[1]);
-    acc[2] = fma(rv, sv, acc[2]);
-    acc[3] = fma(sv, sv, acc[3]);
-    acc[4] = fma(rv, rv, acc[4]);
+    D::add(acc, p[e], sv, D::nd == 3 ? r[e] : 0.0);
   }
-  __shared__ double s_red[(kThreads / 32) * 5];
-  __shared__ double s_sum[5];
-  if (!reduce_last_block<5>(acc, 5, partials, 5, &ctl->counter, s_red, s_sum)) return;
+  __shared__ double s_sum[3];
+  if (!reduce_last_block_fast<D::nd>(acc, partials, &ctl->counter, s_sum)) return;
   if (threadIdx.x != 0) return;
-  base_apply_scalars(ctl, i, slots, mode, s_sum);
+  base_apply_scalars<MODE>(ctl, i, slots, s_sum[0], s_sum[1], s_sum[2]);
 }
 
 // Stencil operators: the same step on the tiled z-marching walk (s = A p and
-// the five dots in its epilogue, r prefetched one plane ahead).
+// the dots in its epilogue, r prefetched one plane ahead where it is read).
+template <int MODE>
 struct BaseApplyEpi {
+  using D = ApplyDots<MODE>;
   double* __restrict__ s;
   const double* __restrict__ r;
-  double acc[5];
+  double acc[D::nd];
   struct Pre {
     double r;
   };
-  __device__ __forceinline__ Pre pre(int64_t c) const { return Pre{r[c]}; }
+  __device__ __forceinline__ Pre pre(int64_t c) const { return Pre{D::nd == 3 ? r[c] : 0.0}; }
   __device__ __forceinline__ void operator()(int64_t c, double sv, double pv, const Pre& p) {
     s[c] = sv;
-    acc[0] = fma(pv, p.r, acc[0]);
-    acc[1] = fma(pv, sv, acc[1]);
-    acc[2] = fma(p.r, sv, acc[2]);
-    acc[3] = fma(sv, sv, acc[3]);
-    acc[4] = fma(p.r, p.r, acc[4]);
+    D::add(acc, pv, sv, p.r);
   }
 };
 
-template <bool ADV>
+template <bool ADV, int MODE>
 __global__ void __launch_bounds__(kTileThreads) base_apply_dots_walk(TiledStencil<double, double> T,
                                                                      double* __restrict__ P, double* __restrict__ S,
                                                                      const double* __restrict__ r, int64_t N,
-                                                                     SolveCtl* ctl, double* partials, int mode) {
+                                                                     SolveCtl* ctl, double* partials) {
   if (ctl->status != kRun) return;
-  const bool fill = (mode == kApplyFcgFill || mode == kApplyGcrFill);
+  constexpr int ND = ApplyDots<MODE>::nd;
+  const bool fill = (MODE == kApplyFcgFill || MODE == kApplyGcrFill);
   const int i = fill ? 0 : ctl->i + 1;
   const int slots = ctl->mmax + 1;
   const size_t off = (size_t)(i % slots) * (size_t)N;
-  BaseApplyEpi e{S + off, r, {0.0, 0.0, 0.0, 0.0, 0.0}};
+  BaseApplyEpi<MODE> e{S + off, r, {}};
   tiled_stencil_walk<double, double, ADV, 1>(T, P + off, e);
-  __shared__ double s_red[(kTileThreads / 32) * 5];
-  __shared__ double s_sum[5];
-  if (!reduce_last_block<5>(e.acc, 5, partials, 5, &ctl->counter, s_red, s_sum)) return;
+  __shared__ double s_sum[3];
+  if (!reduce_last_block_fast<ND>(e.acc, partials, &ctl->counter, s_sum)) return;
   if (threadIdx.x != 0) return;
-  base_apply_scalars(ctl, i, slots, mode, s_sum);
+  base_apply_scalars<MODE>(ctl, i, slots, s_sum[0], s_sum[1], s_sum[2]);
 }
 
 static int base_template(int mmax) { return mmax <= 8 ? 8 : mmax <= 16 ? 16 : 32; }
 
 static cudaError_t launch_window_dots(const SolveEnv& env, int tmpl, const double* v, const double* r,
                                       const double* S, int mode) {
-  const int64_t need = (env.N + kBaseThreads - 1) / kBaseThreads;
-  const int64_t cap = (int64_t)env.ctx->num_sms * kBaseBlocksPerSm;
-  const int blocks = (int)(need < cap ? need : cap);
+  const int blocks = window_dots_blocks(env.ctx, env.N);
   if (!env.partials_fit_2l(blocks, tmpl + 2)) return cudaErrorInvalidValue;
   switch (tmpl) {
-    case 8: base_window_dots<8><<<blocks, kBaseThreads, 0, env.st>>>(v, r, S, env.N, env.ctl, env.partials, mode); break;
-    case 16: base_window_dots<16><<<blocks, kBaseThreads, 0, env.st>>>(v, r, S, env.N, env.ctl, env.partials, mode); break;
-    default: base_window_dots<32><<<blocks, kBaseThreads, 0, env.st>>>(v, r, S, env.N, env.ctl, env.partials, mode); break;
+    case 8: base_window_dots<8><<<blocks, kWinThreads, 0, env.st>>>(v, r, S, env.N, env.ctl, env.partials, mode); break;
+    case 16: base_window_dots<16><<<blocks, kWinThreads, 0, env.st>>>(v, r, S, env.N, env.ctl, env.partials, mode); break;
+    default: base_window_dots<32><<<blocks, kWinThreads, 0, env.st>>>(v, r, S, env.N, env.ctl, env.partials, mode); break;
   }
   return cudaGetLastError();
 }
@@ -301,23 +292,25 @@ static cudaError_t launch_maxpy(const SolveEnv& env, int tmpl, const double* u, 
   return cudaGetLastError();
 }
 
-static cudaError_t launch_apply_dots(const SolveEnv& env, double* P, double* S, const double* r, int mode) {
+template <int MODE>
+static cudaError_t launch_apply_dots(const SolveEnv& env, double* P, double* S, const double* r) {
   const pfk_operator* op = env.op;
+  constexpr int ND = ApplyDots<MODE>::nd;
   if (!op->rowptr) {
     TiledStencil<double, double> T;
     const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
-    const int slots = adv ? tiled_stencil_slots(base_apply_dots_walk<true>, env.ctx->num_sms)
-                          : tiled_stencil_slots(base_apply_dots_walk<false>, env.ctx->num_sms);
+    const int slots = adv ? tiled_stencil_slots(base_apply_dots_walk<true, MODE>, env.ctx->num_sms)
+                          : tiled_stencil_slots(base_apply_dots_walk<false, MODE>, env.ctx->num_sms);
     const int units = tiled_stencil_setup<double, double>(T, op, op->d, op->kx, op->ky, op->kz, slots);
-    const int64_t cap = env.partials_cap / 5;
+    const int64_t cap = env.partials_cap / ND;
     const int blocks = (int)(units < cap ? units : cap);
-    if (adv) base_apply_dots_walk<true><<<blocks, kTileThreads, 0, env.st>>>(T, P, S, r, env.N, env.ctl, env.partials, mode);
-    else base_apply_dots_walk<false><<<blocks, kTileThreads, 0, env.st>>>(T, P, S, r, env.N, env.ctl, env.partials, mode);
+    if (adv) base_apply_dots_walk<true, MODE><<<blocks, kTileThreads, 0, env.st>>>(T, P, S, r, env.N, env.ctl, env.partials);
+    else base_apply_dots_walk<false, MODE><<<blocks, kTileThreads, 0, env.st>>>(T, P, S, r, env.N, env.ctl, env.partials);
     return cudaGetLastError();
   }
   const int blocks = stream_blocks(env.ctx, env.N, 2);
-  if (!env.partials_fit(blocks, 5)) return cudaErrorInvalidValue;
-  base_apply_dots<<<blocks, kThreads, 0, env.st>>>(csr_of(env.op), P, S, r, env.N, env.ctl, env.partials, mode);
+  if (!env.partials_fit(blocks, ND)) return cudaErrorInvalidValue;
+  base_apply_dots<MODE><<<blocks, kThreads, 0, env.st>>>(csr_of(env.op), P, S, r, env.N, env.ctl, env.partials);
   return cudaGetLastError();
 }
 
@@ -342,7 +335,7 @@ class Fcg : public Method {
     cudaError_t e;
     if ((e = op_apply(env.op, x, r_, b, nullptr, env.st)) != cudaSuccess) return e;   // r_0 = b - A x_0
     if ((e = env.pc_apply(r_, P_, nullptr, nullptr)) != cudaSuccess) return e;       // p_0 = u_0 = B(r_0)
-    return launch_apply_dots(env, P_, S_, r_, kApplyFcgFill);                          // s_0 = A p_0, gamma_0, eta_0
+    return launch_apply_dots<kApplyFcgFill>(env, P_, S_, r_);                          // s_0 = A p_0, gamma_0, eta_0
   }
   cudaError_t iteration(const SolveEnv& env, double* x) override {
     if (persistent_) {
@@ -362,7 +355,7 @@ class Fcg : public Method {
     if ((e = env.mark_pass(0)) != cudaSuccess) return e;
     if ((e = launch_window_dots(env, tmpl, u_, r_, S_, kDotsFcg)) != cudaSuccess) return e;   // gamma_i, betas
     if ((e = launch_maxpy(env, tmpl, u_, P_)) != cudaSuccess) return e;                // p_i
-    if ((e = launch_apply_dots(env, P_, S_, r_, kApplyFcgEta)) != cudaSuccess) return e;      // s_i, eta_i, alpha_i
+    if ((e = launch_apply_dots<kApplyFcgEta>(env, P_, S_, r_)) != cudaSuccess) return e;      // s_i, eta_i, alpha_i
     return env.mark_pass(1);
   }
 
@@ -390,7 +383,7 @@ class Gcr : public Method {
     cudaError_t e;
     if ((e = op_apply(env.op, x, r_, b, nullptr, env.st)) != cudaSuccess) return e;   // r_0
     if ((e = env.pc_apply(r_, P_, nullptr, nullptr)) != cudaSuccess) return e;       // p_0 = u_0 = B(r_0)
-    return launch_apply_dots(env, P_, S_, r_, kApplyGcrFill);                          // s_0, gamma_0, eta_0
+    return launch_apply_dots<kApplyGcrFill>(env, P_, S_, r_);                          // s_0, gamma_0, eta_0
   }
   cudaError_t iteration(const SolveEnv& env, double* x) override {
     const int* status = &env.ctl->status;
@@ -403,7 +396,7 @@ class Gcr : public Method {
     if ((e = op_apply(env.op, u_, au_, nullptr, status, env.st)) != cudaSuccess) return e;   // A u_i
     if ((e = launch_window_dots(env, tmpl, au_, r_, S_, kDotsGcr)) != cudaSuccess) return e;  // betas
     if ((e = launch_maxpy(env, tmpl, u_, P_)) != cudaSuccess) return e;                // p_i
-    if ((e = launch_apply_dots(env, P_, S_, r_, kApplyGcrFinal)) != cudaSuccess) return e;    // s_i, gamma, eta
+    if ((e = launch_apply_dots<kApplyGcrFinal>(env, P_, S_, r_)) != cudaSuccess) return e;    // s_i, gamma, eta
     return env.mark_pass(1);
   }
 
@@ -436,9 +429,8 @@ __global__ void __launch_bounds__(kThreads) fgb_fill_norm(const double* __restri
   double acc[1] = {0.0};
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N; e += (int64_t)gridDim.x * blockDim.x)
     acc[0] = fma(r[e], r[e], acc[0]);
-  __shared__ double s_red[kThreads / 32];
   __shared__ double s_sum[1];
-  if (!reduce_last_block<1>(acc, 1, partials, 1, &ctl->counter, s_red, s_sum)) return;
+  if (!reduce_last_block_fast<1>(acc, partials, &ctl->counter, s_sum)) return;
   if (threadIdx.x != 0) return;
   const double beta = sqrt(s_sum[0]);
   if (!ctl->target_set) {
@@ -525,53 +517,29 @@ static cudaError_t launch_apply_store(const SolveEnv& env, const double* ucur, d
   return cudaGetLastError();
 }
 
-// Classical Gram-Schmidt coefficients h_{j,k} = <p_j, z_k>, j <= k (transposed dots).
+// Classical Gram-Schmidt coefficients h_{j,k} = <p_j, z_k>, j <= k (window_dots).
 template <int NW>
-__global__ void __launch_bounds__(kBaseThreads, kBaseBlocksPerSm) fgb_dots(const double* __restrict__ z,
-                                                                           const double* __restrict__ P, int64_t N,
-                                                                           SolveCtl* ctl, FgState* gs,
-                                                                           double* partials) {
+__global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) fgb_dots(const double* __restrict__ z,
+                                                                         const double* __restrict__ P, int64_t N,
+                                                                         SolveCtl* ctl, FgState* gs,
+                                                                         double* partials) {
   if (ctl->status != kRun) return;
   constexpr int ND = NW;
-  constexpr int NWARPS = kBaseThreads / 32;
-  __shared__ double s_pk[NW * kBaseStride];
-  __shared__ double s_z[kBaseThreads];
+  constexpr int NWARPS = kWinThreads / 32;
+  __shared__ size_t s_off[NW];
   __shared__ double s_red[NWARPS * ND];
   __shared__ double s_sum[ND];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nk = gs->k + 1;           // p_0 .. p_k
-  double* my = s_pk + threadIdx.x;
-  const double* wz = s_z + warp * 32;
-  const double* lrow = s_pk + lane * kBaseStride + warp * 32;
-  double gw = 0.0;
-  for (int64_t base = (int64_t)blockIdx.x * kBaseThreads; base < N; base += (int64_t)gridDim.x * kBaseThreads) {
-    const int64_t e = base + threadIdx.x;
-    double zv = 0.0;
-    if (e < N) {
-      zv = z[e];
-#pragma unroll
-      for (int j = 0; j < NW; ++j)
-        if (j < nk) my[j * kBaseStride] = P[(size_t)j * (size_t)N + e];
-    } else {
-#pragma unroll
-      for (int j = 0; j < NW; ++j)
-        if (j < nk) my[j * kBaseStride] = 0.0;
-    }
-    s_z[threadIdx.x] = zv;
-    __syncwarp();
-    if (lane < nk) {
-      double c = gw;
-#pragma unroll 8
-      for (int t = 0; t < 32; ++t) c = fma(wz[t], lrow[t], c);
-      gw = c;
-    }
-    __syncwarp();
-  }
-  if (lane < nk) s_red[warp * nk + lane] = gw;
+  if (threadIdx.x < nk) s_off[threadIdx.x] = (size_t)threadIdx.x * (size_t)N;
+  __syncthreads();
+  double acc[NW];
+  window_dots<NW>(z, P, s_off, nk, N, acc, [](int64_t, double) {});
+  const double tot = warp_sum_transposed<NW>(acc);
+  if (lane < nk) s_red[warp * nk + lane] = tot;
   __syncthreads();
   if (!combine_block_partials_2l(s_red, nk, partials, ND, &ctl->counter, ctl->gcounter, s_sum)) return;
-  if (threadIdx.x != 0) return;
-  for (int j = 0; j < nk; ++j) gs->H[j * kGm + gs->k] = s_sum[j];
+  if ((int)threadIdx.x < nk) gs->H[threadIdx.x * kGm + gs->k] = s_sum[threadIdx.x];
 }
 
 // pbar = z_k - sum_j h_{j,k} p_j into slot k+1, and ||pbar||^2; the last block
@@ -595,39 +563,52 @@ __global__ void __launch_bounds__(kThreads, 3) fgb_orth(const double* __restrict
     if (k + 1 < m) P[out + e] = v;
     acc[0] = fma(v, v, acc[0]);
   }
-  __shared__ double s_red[kThreads / 32];
   __shared__ double s_sum[1];
-  if (!reduce_last_block<1>(acc, 1, partials, 1, &ctl->counter, s_red, s_sum)) return;
-  if (threadIdx.x != 0) return;
-  const double h = sqrt(s_sum[0]);
-  gs->H[(k + 1) * kGm + k] = h;
-  ctl->it += 1;
-  gs->ncols = k + 1;
-  ctl->i = k + 1;
-  for (int j = 0; j <= k + 1; ++j) gs->R[j * kGm + k] = gs->H[j * kGm + k];
-  for (int j = 0; j < k; ++j) {
-    const double a = gs->R[j * kGm + k], b = gs->R[(j + 1) * kGm + k];
-    gs->R[j * kGm + k] = gs->cs[j] * a + gs->sn[j] * b;
-    gs->R[(j + 1) * kGm + k] = -gs->sn[j] * a + gs->cs[j] * b;
+  if (!reduce_last_block_fast<1>(acc, partials, &ctl->counter, s_sum)) return;
+  // column k in shared memory: the rotations are loaded and the column stored
+  // by the block's threads, thread 0 runs the recurrence
+  __shared__ double s_cs[NW], s_sn[NW], s_r[NW + 1];
+  if ((int)threadIdx.x < nk) {
+    s_r[threadIdx.x] = s_h[threadIdx.x];
+    if ((int)threadIdx.x < k) {
+      s_cs[threadIdx.x] = gs->cs[threadIdx.x];
+      s_sn[threadIdx.x] = gs->sn[threadIdx.x];
+    }
   }
-  const double a = gs->R[k * kGm + k], b = gs->R[(k + 1) * kGm + k];
-  const double rr = hypot(a, b);
-  const double c = rr != 0.0 ? a / rr : 1.0, s = rr != 0.0 ? b / rr : 0.0;
-  gs->cs[k] = c;
-  gs->sn[k] = s;
-  gs->R[k * kGm + k] = rr;
-  gs->R[(k + 1) * kGm + k] = 0.0;
-  gs->g[k + 1] = -s * gs->g[k];
-  gs->g[k] = c * gs->g[k];
-  const double est = fabs(gs->g[k + 1]);
-  ctl->rho = est;
-  push_history(ctl, est, nan(""), nan(""), h);
-  gs->inv = h != 0.0 ? 1.0 / h : 0.0;
-  gs->k = k + 1;
-  if (!isfinite(est)) { ctl->status = kNonFinite; return; }
-  if (est <= ctl->target || h == 0.0) { ctl->status = kConverged; return; }
-  if (k + 1 == m) { ctl->status = kCycleEnd; return; }
-  if (ctl->it >= ctl->maxit) { ctl->status = kMaxit; return; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double h = sqrt(s_sum[0]);
+    gs->H[(k + 1) * kGm + k] = h;
+    ctl->it += 1;
+    gs->ncols = k + 1;
+    ctl->i = k + 1;
+    double a = s_r[0];
+    for (int j = 0; j < k; ++j) {
+      const double b = s_r[j + 1];
+      s_r[j] = s_cs[j] * a + s_sn[j] * b;
+      a = -s_sn[j] * a + s_cs[j] * b;
+    }
+    const double rr = hypot(a, h);
+    const double c = rr != 0.0 ? a / rr : 1.0, s = rr != 0.0 ? h / rr : 0.0;
+    gs->cs[k] = c;
+    gs->sn[k] = s;
+    s_r[k] = rr;
+    gs->R[(k + 1) * kGm + k] = 0.0;
+    const double gk = gs->g[k];
+    gs->g[k + 1] = -s * gk;
+    gs->g[k] = c * gk;
+    const double est = fabs(-s * gk);
+    ctl->rho = est;
+    push_history(ctl, est, nan(""), nan(""), h);
+    gs->inv = h != 0.0 ? 1.0 / h : 0.0;
+    gs->k = k + 1;
+    if (!isfinite(est)) ctl->status = kNonFinite;
+    else if (est <= ctl->target || h == 0.0) ctl->status = kConverged;
+    else if (k + 1 == m) ctl->status = kCycleEnd;
+    else if (ctl->it >= ctl->maxit) ctl->status = kMaxit;
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < nk) gs->R[threadIdx.x * kGm + k] = s_r[threadIdx.x];
 }
 
 __global__ void fgb_lsq(FgState* gs) {
@@ -684,24 +665,22 @@ class Fgmres : public Method {
     (void)x;
     const int* status = &env.ctl->status;
     const int tmpl = base_template(m_ + 1);
-    const int64_t need = (N_ + kBaseThreads - 1) / kBaseThreads;
-    const int64_t cap = (int64_t)env.ctx->num_sms * kBaseBlocksPerSm;
-    const int dblocks = (int)(need < cap ? need : cap);
+    const int dblocks = window_dots_blocks(env.ctx, N_);
     const int oblocks = stream_blocks(env.ctx, N_, 2);
     if (!env.partials_fit_2l(dblocks, tmpl) || !env.partials_fit(oblocks, 1)) return cudaErrorInvalidValue;
     cudaError_t e;
     if ((e = env.mark_pass(0)) != cudaSuccess) return e;
     switch (tmpl) {
       case 8:
-        fgb_dots<8><<<dblocks, kBaseThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, env.partials);
+        fgb_dots<8><<<dblocks, kWinThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, env.partials);
         fgb_orth<8><<<oblocks, kThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, m_, env.partials);
         break;
       case 16:
-        fgb_dots<16><<<dblocks, kBaseThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, env.partials);
+        fgb_dots<16><<<dblocks, kWinThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, env.partials);
         fgb_orth<16><<<oblocks, kThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, m_, env.partials);
         break;
       default:
-        fgb_dots<32><<<dblocks, kBaseThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, env.partials);
+        fgb_dots<32><<<dblocks, kWinThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, env.partials);
         fgb_orth<32><<<oblocks, kThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, m_, env.partials);
         break;
     }

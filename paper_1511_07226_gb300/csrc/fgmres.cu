@@ -60,54 +60,74 @@ struct FgArgs {
 };
 
 // Column k of H from its dots (hb[j] = <p_j, zbar_k>, j <= k; zz = ||zbar_k||^2),
-// Givens update and status.  One thread.
-__device__ void fgmres_column(SolveCtl* ctl, GmresState* gs, int k, int m, const double* hb, double zz) {
+// Givens update and status.  All threads of the (last) block: they load the
+// rotations and store the column; thread 0 runs the recurrences on shared
+// memory in column order (on the column in global memory each rotation waited
+// for two L2 round trips).  s_tmp: 3 kGm + 2 doubles of shared memory.
+__device__ void fgmres_column(SolveCtl* ctl, GmresState* gs, int k, int m, const double* hb, double zz,
+                              double* s_tmp) {
+  double* s_cs = s_tmp;
+  double* s_sn = s_tmp + kGm;
+  double* s_r = s_tmp + 2 * kGm;        // kGm + 2: the column, and whether it is valid
   const double sigma = gs->sigma;
-  double tsum = 0.0;
-  for (int j = 0; j <= k; ++j) {
+  for (int j = threadIdx.x; j <= k; j += blockDim.x) {
+    const double h = j == k ? hb[j] + sigma : hb[j];
     gs->Hb[j * kGm + k] = hb[j];
-    gs->H[j * kGm + k] = hb[j];
-    tsum += hb[j] * hb[j];
+    gs->H[j * kGm + k] = h;
+    s_r[j] = h;
+    if (j < k) {
+      s_cs[j] = gs->cs[j];
+      s_sn[j] = gs->sn[j];
+    }
   }
-  gs->H[k * kGm + k] = hb[k] + sigma;
-  const double t = zz - tsum;
-  if (!(t >= 0.0)) {
-    ctl->i = k + 1;     // breakdown while forming column k: columns 0 .. k-1 valid
-    gs->ncols = k;
-    ctl->status = isfinite(t) ? kBreakdown : kNonFinite;
-    return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_r[kGm + 1] = 0.0;
+    double tsum = 0.0;
+    for (int j = 0; j <= k; ++j) tsum += hb[j] * hb[j];
+    const double t = zz - tsum;
+    if (!(t >= 0.0)) {
+      ctl->i = k + 1;     // breakdown while forming column k: columns 0 .. k-1 valid
+      gs->ncols = k;
+      ctl->status = isfinite(t) ? kBreakdown : kNonFinite;
+    } else {
+      s_r[kGm + 1] = 1.0;
+      const double hsub = sqrt(t);
+      gs->Hb[(k + 1) * kGm + k] = hsub;
+      gs->H[(k + 1) * kGm + k] = hsub;
+      ctl->it += 1;
+      gs->ncols = k + 1;
+      ctl->i = k + 1;
+      // Givens: apply the previous rotations to column k, then zero its subdiagonal
+      double a = s_r[0];
+      for (int j = 0; j < k; ++j) {
+        const double b = s_r[j + 1];
+        s_r[j] = s_cs[j] * a + s_sn[j] * b;
+        a = -s_sn[j] * a + s_cs[j] * b;
+      }
+      const double rr = hypot(a, hsub);
+      const double c = rr != 0.0 ? a / rr : 1.0, sn = rr != 0.0 ? hsub / rr : 0.0;
+      gs->cs[k] = c;
+      gs->sn[k] = sn;
+      s_r[k] = rr;
+      gs->R[(k + 1) * kGm + k] = 0.0;
+      const double gk = gs->g[k];
+      gs->g[k + 1] = -sn * gk;
+      gs->g[k] = c * gk;
+      const double est = fabs(-sn * gk);
+      ctl->rho = est;
+      push_history(ctl, est, nan(""), t, hsub);
+      gs->inv = hsub != 0.0 ? 1.0 / hsub : 0.0;
+      gs->k = k + 1;
+      if (!isfinite(est)) ctl->status = kNonFinite;
+      else if (est <= ctl->target || t == 0.0) ctl->status = kConverged;
+      else if (k + 1 == m) ctl->status = kCycleEnd;
+      else if (ctl->it >= ctl->maxit) ctl->status = kMaxit;
+    }
   }
-  const double hsub = sqrt(t);
-  gs->Hb[(k + 1) * kGm + k] = hsub;
-  gs->H[(k + 1) * kGm + k] = hsub;
-  ctl->it += 1;
-  gs->ncols = k + 1;
-  ctl->i = k + 1;
-  // Givens: apply the previous rotations to column k, then zero its subdiagonal
-  for (int j = 0; j <= k + 1; ++j) gs->R[j * kGm + k] = gs->H[j * kGm + k];
-  for (int j = 0; j < k; ++j) {
-    const double a = gs->R[j * kGm + k], b = gs->R[(j + 1) * kGm + k];
-    gs->R[j * kGm + k] = gs->cs[j] * a + gs->sn[j] * b;
-    gs->R[(j + 1) * kGm + k] = -gs->sn[j] * a + gs->cs[j] * b;
-  }
-  const double a = gs->R[k * kGm + k], b = gs->R[(k + 1) * kGm + k];
-  const double rr = hypot(a, b);
-  const double c = rr != 0.0 ? a / rr : 1.0, s = rr != 0.0 ? b / rr : 0.0;
-  gs->cs[k] = c;
-  gs->sn[k] = s;
-  gs->R[k * kGm + k] = rr;
-  gs->R[(k + 1) * kGm + k] = 0.0;
-  gs->g[k + 1] = -s * gs->g[k];
-  gs->g[k] = c * gs->g[k];
-  const double est = fabs(gs->g[k + 1]);
-  ctl->rho = est;
-  push_history(ctl, est, nan(""), t, hsub);
-  gs->inv = hsub != 0.0 ? 1.0 / hsub : 0.0;
-  gs->k = k + 1;
-  if (!isfinite(est)) { ctl->status = kNonFinite; return; }
-  if (est <= ctl->target || t == 0.0) { ctl->status = kConverged; return; }
-  if (k + 1 == m) { ctl->status = kCycleEnd; return; }
-  if (ctl->it >= ctl->maxit) { ctl->status = kMaxit; return; }
+  __syncthreads();
+  if (s_r[kGm + 1] != 0.0)
+    for (int j = threadIdx.x; j <= k; j += blockDim.x) gs->R[j * kGm + k] = s_r[j];
 }
 
 constexpr int kFgThreads = 128;
@@ -194,13 +214,15 @@ __global__ void __launch_bounds__(kFgThreads, kFgBlocksPerSm) fgmres_pass(FgArgs
     __syncthreads();
   }
   if (!combine_block_partials_2l(s_red, k + 2, a.partials, ND, &ctl->counter, ctl->gcounter, s_sum)) return;
-  if (threadIdx.x != 0) return;
-  // traffic: zbar_{k-1}, qbar, wbar and 3k window vectors read, p_k, u_k,
-  // zbar_k written; FP64: 3k MAXPY FMAs, 3 scalings, k + 2 dot FMAs
-  ctl->passes += 1;
-  ctl->alg_bytes += 8.0 * (double)N * (double)(3 + 3 * k + 4);
-  ctl->alg_flops += (double)N * (2.0 * (3 * k + k + 2) + 3.0);
-  fgmres_column(ctl, gs, k, a.m, s_sum + 1, s_sum[0]);
+  if (threadIdx.x == 0) {
+    // traffic: zbar_{k-1}, qbar, wbar and 3k window vectors read, p_k, u_k,
+    // zbar_k written; FP64: 3k MAXPY FMAs, 3 scalings, k + 2 dot FMAs
+    ctl->passes += 1;
+    ctl->alg_bytes += 8.0 * (double)N * (double)(3 + 3 * k + 4);
+    ctl->alg_flops += (double)N * (2.0 * (3 * k + k + 2) + 3.0);
+  }
+  static_assert(NW * kFgStride >= 3 * kGm + 2, "the column's scratch fits in the parked p_j");
+  fgmres_column(ctl, gs, k, a.m, s_sum + 1, s_sum[0], s_pk);
 }
 
 // beta = ||r_0||: history, target, convergence; g = beta e_0.
@@ -259,8 +281,8 @@ __global__ void __launch_bounds__(kThreads) fgmres_fill_col0(const double* __res
   __shared__ double s_red[(kThreads / 32) * 2];
   __shared__ double s_sum[2];
   if (!reduce_last_block<2>(acc, 2, partials, 2, &ctl->counter, s_red, s_sum)) return;
-  if (threadIdx.x != 0) return;
-  fgmres_column(ctl, gs, 0, m, s_sum + 1, s_sum[0]);
+  __shared__ double s_tmp[3 * kGm + 2];
+  fgmres_column(ctl, gs, 0, m, s_sum + 1, s_sum[0], s_tmp);
 }
 
 // End of a cycle: back substitution R y = g on the ncols valid columns.

@@ -232,25 +232,21 @@ __global__ void __launch_bounds__(kTileThreads) pipegcr_apply_walk(TiledStencil<
   GcrApplyEpi e{a.w, a.t, a.r, 0.0, 0.0, 0.0};
   tiled_stencil_walk<double, double, ADV, 1>(T, a.u, e);
   double acc[3] = {e.g0, e.g1, e.g2};
-  __shared__ double smem[(kTileThreads / 32) * 3];
   __shared__ double sums[3];
-  if (reduce_last_block<3>(acc, 3, a.partials, 3, &ctl->counter, smem, sums) && threadIdx.x == 0) {
+  if (reduce_last_block_fast<3>(acc, a.partials, &ctl->counter, sums) && threadIdx.x == 0) {
     ctl->pend[0] = sums[0];
     ctl->pend[1] = sums[1];
     ctl->pend[2] = sums[2];
   }
 }
 
-// <w_i, s_k> over the window, one register accumulator per window slot and
-// thread (independent FMAs, no shared-memory staging); the last block adds the
+// <w_i, s_k> over the window (window_dots); the last block adds the
 // walk's gamma, delta, ||r||^2 and runs the scalar phase of iteration i.
-constexpr int kWinBlocksPerSm = 5;   // 93 registers at NW = 32
-
 template <int NW>
-__global__ void __launch_bounds__(kGcrThreads, kWinBlocksPerSm) pipegcr_window_dots(GcrArgs a, int stencil_flops) {
+__global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) pipegcr_window_dots(GcrArgs a, int stencil_flops) {
   SolveCtl* ctl = a.ctl;
   if (ctl->status != kRun) return;
-  constexpr int NWARPS = kGcrThreads / 32;
+  constexpr int NWARPS = kWinThreads / 32;
   __shared__ size_t s_off[NW];
   __shared__ double s_red[NWARPS * NW];
   __shared__ double s_sum[NW];
@@ -265,21 +261,9 @@ __global__ void __launch_bounds__(kGcrThreads, kWinBlocksPerSm) pipegcr_window_d
   }
   __syncthreads();
   double acc[NW];
-#pragma unroll
-  for (int j = 0; j < NW; ++j) acc[j] = 0.0;
-  for (int64_t e = (int64_t)blockIdx.x * kGcrThreads + threadIdx.x; e < N; e += (int64_t)gridDim.x * kGcrThreads) {
-    const double wv = __ldg(&a.w[e]);
-#pragma unroll
-    for (int j = 0; j < NW; ++j)
-      if (j < nu) acc[j] = fma(wv, __ldg(&a.S[s_off[j] + e]), acc[j]);
-  }
-#pragma unroll
-  for (int j = 0; j < NW; ++j) {
-    if (j < nu) {
-      const double v = warp_sum(acc[j]);
-      if (lane == 0) s_red[warp * nu + j] = v;
-    }
-  }
+  window_dots<NW>(a.w, a.S, s_off, nu, N, acc, [](int64_t, double) {});
+  const double tot = warp_sum_transposed<NW>(acc);
+  if (lane < nu) s_red[warp * nu + lane] = tot;
   __syncthreads();
   if (!combine_block_partials_2l(s_red, nu, a.partials, NW, &ctl->counter, ctl->gcounter, s_sum)) return;
   if (threadIdx.x == 0) {
@@ -307,9 +291,8 @@ __global__ void __launch_bounds__(kThreads) pipegcr_fill_dots(const double* __re
     acc[1] = fma(wv, wv, acc[1]);
     acc[2] = fma(rv, rv, acc[2]);
   }
-  __shared__ double s_red[(kThreads / 32) * 3];
   __shared__ double s_sum[3];
-  if (!reduce_last_block<3>(acc, 3, partials, 3, &ctl->counter, s_red, s_sum)) return;
+  if (!reduce_last_block_fast<3>(acc, partials, &ctl->counter, s_sum)) return;
   if (threadIdx.x != 0) return;
   cgcr_fill_scalars(ctl, s_sum[0], s_sum[1], s_sum[2]);
 }
@@ -370,9 +353,7 @@ class PipeGcr : public Method {
       const int units = tiled_stencil_setup<double, double>(T, op, op->d, op->kx, op->ky, op->kz, slots);
       const int64_t wcap = env.partials_cap / 3;
       const int wblocks = (int)(units < wcap ? units : wcap);
-      const int64_t wneed = (N_ + kGcrThreads - 1) / kGcrThreads;
-      const int64_t wslots = (int64_t)env.ctx->num_sms * kWinBlocksPerSm;
-      const int sblocks = (int)(wneed < wslots ? wneed : wslots);
+      const int sblocks = window_dots_blocks(env.ctx, N_);
       if (!env.partials_fit_2l(sblocks, tmpl)) return cudaErrorInvalidValue;
       switch (tmpl) {
         case 8: pipegcr_advance<8><<<ablocks, kThreads, 0, env.st>>>(a); break;
@@ -383,9 +364,9 @@ class PipeGcr : public Method {
       else pipegcr_apply_walk<false><<<wblocks, kTileThreads, 0, env.st>>>(T, a);
       const int sf = adv ? 10 : 7;
       switch (tmpl) {
-        case 8: pipegcr_window_dots<8><<<sblocks, kGcrThreads, 0, env.st>>>(a, sf); break;
-        case 16: pipegcr_window_dots<16><<<sblocks, kGcrThreads, 0, env.st>>>(a, sf); break;
-        default: pipegcr_window_dots<32><<<sblocks, kGcrThreads, 0, env.st>>>(a, sf); break;
+        case 8: pipegcr_window_dots<8><<<sblocks, kWinThreads, 0, env.st>>>(a, sf); break;
+        case 16: pipegcr_window_dots<16><<<sblocks, kWinThreads, 0, env.st>>>(a, sf); break;
+        default: pipegcr_window_dots<32><<<sblocks, kWinThreads, 0, env.st>>>(a, sf); break;
       }
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       if ((e = env.mark_pass(1)) != cudaSuccess) return e;

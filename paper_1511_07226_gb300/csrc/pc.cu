@@ -135,6 +135,19 @@ __global__ void __launch_bounds__(kThreads) noisy_row_norms_kernel(const double*
 // Inner Jacobi-PCG
 // ---------------------------------------------------------------------------
 
+// The reductions of the inner PCG: the FP32 form keeps the order its results
+// were pinned with.
+template <typename V>
+__device__ __forceinline__ bool pcg_reduce(const double (&acc)[1], double* partials, unsigned int* counter,
+                                           double* sums) {
+  if constexpr (std::is_same<V, double>::value) {
+    return reduce_last_block_fast<1>(acc, partials, counter, sums);
+  } else {
+    __shared__ double smem[kThreads / 32];
+    return reduce_last_block<1>(acc, 1, partials, 1, counter, smem, sums);
+  }
+}
+
 // A_0 and B_0 in one launch (neither needs the other's result):
 // r_0 = v (not stored: A_1 reads v), p_0 = D^-1 r_0, gamma_0 = <D^-1 r_0, r_0>;
 // finalize: stop at once (B(v) = 0) if gamma_0 == 0 (then v and p_0 are zero).
@@ -151,9 +164,8 @@ __global__ void __launch_bounds__(kThreads) pcg_first_kernel(StencilT<V, C> A, c
     accv += z * rv;
   }
   double acc[1] = {(double)accv};
-  __shared__ double smem[kThreads / 32];
   __shared__ double sums[1];
-  if (reduce_last_block<1>(acc, 1, partials, 1, &ctl->counter, smem, sums) && threadIdx.x == 0) {
+  if (pcg_reduce<V>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0) {
     const double g = sums[0];
     ctl->gamma = g;
     ctl->ok = (g == 0.0) ? 0 : k;
@@ -171,15 +183,27 @@ __global__ void __launch_bounds__(kThreads) pcg_a_kernel(StencilT<V, C> A, const
   if (i > last_x) return;
   const V alpha = (V)ctl->alpha[i - 1];
   V accv = V(0);
-  GRID_LOOP(c, A.n) {
+  const int64_t T = (int64_t)gridDim.x * blockDim.x;
+  int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  // FP64: two cells' loads in flight, added in order (half the blocks of the FP32 form)
+  for (; std::is_same<V, double>::value && c + T < A.n; c += 2 * T) {
+    const V r0 = i == 1 ? (V)v[c] : r[c], r1 = i == 1 ? (V)v[c + T] : r[c + T];
+    const V s0 = s[c], s1 = s[c + T];
+    const V d0 = cv<V, C>(A.dinv[c]), d1 = cv<V, C>(A.dinv[c + T]);
+    const V n0 = r0 - alpha * s0, n1 = r1 - alpha * s1;
+    r[c] = n0;
+    r[c + T] = n1;
+    accv += (d0 * n0) * n0;
+    accv += (d1 * n1) * n1;
+  }
+  for (; c < A.n; c += T) {
     const V rv = (i == 1 ? (V)v[c] : r[c]) - alpha * s[c];
     r[c] = rv;
     accv += (cv<V, C>(A.dinv[c]) * rv) * rv;
   }
   double acc[1] = {(double)accv};
-  __shared__ double smem[kThreads / 32];
   __shared__ double sums[1];
-  if (reduce_last_block<1>(acc, 1, partials, 1, &ctl->counter, smem, sums) && threadIdx.x == 0) {
+  if (pcg_reduce<V>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0) {
     const double g = sums[0];
     if (g == 0.0) {
       ctl->ok = i;
@@ -233,9 +257,8 @@ __global__ void __launch_bounds__(kTileThreads) pcg_c_kernel(TiledStencil<V, C> 
   PcgCEpi<V> e{s, V(0)};
   tiled_stencil_walk<V, C, ADV, tiled_width<V, C>()>(T, p, e);
   double acc[1] = {(double)e.acc};
-  __shared__ double smem[kTileThreads / 32];
   __shared__ double sums[1];
-  if (reduce_last_block<1>(acc, 1, partials, 1, &ctl->counter, smem, sums) && threadIdx.x == 0) {
+  if (pcg_reduce<V>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0) {
     const double eta = sums[0];
     if (eta == 0.0) {
       ctl->ok = i;
@@ -455,7 +478,10 @@ static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v
   V* x = base + 2 * n;
   V* p[2] = {base + 3 * n, base + 4 * n};
   const int k = pc->inner;
-  const int blocks = stream_blocks(pc->ctx, n, 8);
+  // reducing kernels: 4 blocks per SM in FP64 (every block adds 12 FP64
+  // instructions to the sum), 8 in FP32, where the FP32 partial sums of a
+  // thread fix the grid
+  const int blocks = stream_blocks(pc->ctx, n, std::is_same<V, double>::value ? 4 : 8);
   const int sblocks = stream_blocks(pc->ctx, n, 8);
   TiledStencil<V, C> T;
   const pfk_operator* op = pc->op;

@@ -200,6 +200,53 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sums V values of every lane over the warp (V a power of two, at most 32):
+// lane l returns the sum of acc[l % V].  Each step exchanges half of the
+// values a lane still holds with a partner lane, so the warp spends V - 1 (+
+// 5 - log2 V) FP64 additions instead of the 5 V of V shuffle trees: on GB300
+// an FP64 warp instruction holds its pipe for ~76 cycles, and the 160
+// additions of 32 trees cost a resident warp as much as the products of five
+// elements.
+template <int V>
+__device__ __forceinline__ double warp_sum_transposed(double (&acc)[V]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = V / 2; h > 0; h >>= 1) {
+    const bool up = (lane & h) != 0;
+#pragma unroll
+    for (int j = 0; j < h; ++j) {
+      const double keep = up ? acc[j + h] : acc[j], send = up ? acc[j] : acc[j + h];
+      acc[j] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+    }
+  }
+  double v = acc[0];
+#pragma unroll
+  for (int o = V; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Value j of every thread summed over the block (ND values of kThreads
+// threads, staged in buf): warp (blockIdx + j) mod 8 adds the eight warps'
+// values lane by lane and runs one shuffle tree, so a value costs the block 12
+// FP64 instructions instead of 8 trees of 5; the warp rotates with the block
+// so that the resident blocks' sums spread over the SM's four FP64 pipes.
+// store(j, sum) is called by lane 0 of that warp.
+template <int ND, typename F>
+__device__ __forceinline__ void block_sums(const double (&acc)[ND], double (&buf)[ND][kThreads], F&& store) {
+  static_assert(ND <= kThreads / 32 && kThreads == 256, "one warp per value, eight warps");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int j = 0; j < ND; ++j) buf[j][threadIdx.x] = acc[j];
+  __syncthreads();
+  const int j = (warp - (int)blockIdx.x) & 7;
+  if (j < ND) {
+    const double* b = buf[j] + lane;
+    const double v = ((b[0] + b[64]) + (b[128] + b[192])) + ((b[32] + b[96]) + (b[160] + b[224]));
+    const double w = warp_sum(v);
+    if (lane == 0) store(j, w);
+  }
+}
+
 // sums over rows: out[j] = sum_{b < nrows} rows[b * stride + j], j < nd, by
 // all threads of the block.  The loads come from L2 (~0.4 us each) while the
 // rest of the GPU may idle, so they are issued many at a time: for nd <= 4
@@ -361,6 +408,44 @@ __device__ __forceinline__ bool reduce_last_block(const double (&acc)[ND], int n
   }
   __syncthreads();
   return combine_block_partials(smem, nd, partials, stride, counter, sums);
+}
+
+// reduce_last_block for the kernels of the FP64 path (blocks of kThreads
+// threads), with block_sums in place of the shuffle trees: partials[blockIdx.x *
+// ND + j]; the last block's thread t takes rows t, t + kThreads, ..., then
+// block_sums.  At 64^3 the inner PCG's r update went from 9.0 to 5.6 us and
+// s = A p from 10.2 to 8.8 us, most of it the trees of 64 resident warps.  The
+// reductions that also serve the reduced-precision preconditioners and
+// PIPEFGMRES's shift keep reduce_last_block: a last-bit change there moves
+// FP32 roundings downstream.
+template <int ND>
+__device__ __forceinline__ bool reduce_last_block_fast(const double (&acc)[ND], double* partials, unsigned int* counter,
+                                                  double* sums) {
+  __shared__ double buf[ND][kThreads];
+  block_sums<ND>(acc, buf, [&](int j, double v) { partials[(size_t)blockIdx.x * ND + j] = v; });
+  if (!arrive_last(counter, gridDim.x)) return false;
+  double t[ND];
+#pragma unroll
+  for (int j = 0; j < ND; ++j) t[j] = 0.0;
+  const int nrows = gridDim.x;
+  constexpr int U = ND == 1 ? 8 : 4;   // rows in flight per thread
+  for (int b = threadIdx.x; b < nrows; b += U * kThreads) {
+    double q[U][ND];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int j = 0; j < ND; ++j)
+        q[u][j] = b + u * kThreads < nrows ? __ldcg(&partials[(size_t)(b + u * kThreads) * ND + j]) : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (u == 0 || b + u * kThreads < nrows)
+#pragma unroll
+        for (int j = 0; j < ND; ++j) t[j] += q[u][j];
+  }
+  block_sums<ND>(t, buf, [&](int j, double v) { sums[j] = v; });
+  __syncthreads();
+  if (threadIdx.x == 0) *counter = 0u;
+  return true;
 }
 
 // ---------------------------------------------------------------------------

@@ -66,6 +66,39 @@ class Method {
   }
 };
 
+// Window dots, the reduction of the CR types and the base methods: one
+// register accumulator per window slot and thread (independent FMAs, the
+// loads of a whole window in flight), then warp_sum_transposed.  acc[j] +=
+// <v, s_j> over the elements e = first, first + step, ...; s_off holds the
+// slots' offsets.  body(e, v_e) adds the caller's own products.
+constexpr int kWinThreads = 128;
+constexpr int kWinBlocksPerSm = 5;   // 93 registers at NW = 32
+
+template <int NW, typename F>
+__device__ __forceinline__ void window_dots(const double* __restrict__ v, const double* __restrict__ S,
+                                            const size_t* s_off, int nu, int64_t N, double (&acc)[NW], F&& body) {
+#pragma unroll
+  for (int j = 0; j < NW; ++j) acc[j] = 0.0;
+  for (int64_t e = (int64_t)blockIdx.x * kWinThreads + threadIdx.x; e < N; e += (int64_t)gridDim.x * kWinThreads) {
+    const double ve = __ldg(&v[e]);
+#pragma unroll
+    for (int j = 0; j < NW; ++j)
+      if (j < nu) acc[j] = fma(ve, __ldg(&S[s_off[j] + e]), acc[j]);
+    body(e, ve);
+  }
+}
+
+// Grid of a window-dots kernel: four elements per thread once that still fills
+// the GPU with two blocks per SM (the tail of 31 FP64 additions per warp is
+// shared by more products), fewer below, and at most kWinBlocksPerSm blocks
+// per SM.
+inline int window_dots_blocks(const pfk_context* ctx, int64_t N) {
+  const int64_t cap = (int64_t)ctx->num_sms * kWinBlocksPerSm, two = (int64_t)ctx->num_sms * 2;
+  const int64_t one = (N + kWinThreads - 1) / kWinThreads, four = (N + 4 * kWinThreads - 1) / (4 * kWinThreads);
+  const int64_t b = four >= two ? four : (one < two ? one : two);
+  return (int)(b < cap ? b : cap);
+}
+
 // Persistent single-launch iterations (persistent.cu): eligibility, and one
 // cooperative launch of up to `iters` PIPEFCG (pipelined) or FCG iterations.
 // FCG passes w, m0, m1, n, Q, Z as null.
