@@ -85,7 +85,7 @@ pfk_status pfk_create_context(int device, void* cuda_stream, pfk_context** out) 
     pfk_destroy_context(ctx);
     return cuda_fail(nullptr, e, "cudaStreamCreate (capture stream)");
   }
-  if ((e = cudaMallocHost((void**)&ctx->pinned, 2 * sizeof(SolveCtl))) != cudaSuccess) {
+  if ((e = cudaMallocHost((void**)&ctx->pinned, 2 * sizeof(SolveCtl) + 2 * sizeof(double))) != cudaSuccess) {
     pfk_destroy_context(ctx);
     return cuda_fail(nullptr, e, "cudaMallocHost (status words)");
   }

@@ -107,7 +107,7 @@ struct pfk_context {
   double* scratch_partials = nullptr;   // reduction partials for standalone calls
   unsigned int* scratch_counter = nullptr;
   double* scratch_out = nullptr;
-  pfk::SolveCtl* pinned = nullptr;      // host-pinned status copies of pfk_solve
+  pfk::SolveCtl* pinned = nullptr;      // host-pinned: two status copies of pfk_solve and two scalars
   // block sizes autotuned by pfk_solve_batched, keyed by (mmax template, log2 of
   // the largest system, count bucket, preconditioner precision + 2 x inner iterations)
   std::map<std::tuple<int, int, int, int>, int> batched_tuned;

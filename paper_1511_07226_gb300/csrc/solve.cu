@@ -2,12 +2,18 @@
 //
 // Host logic only (scalars and control); every vector operation is a kernel of
 // the method object.  Per solve:
-//   1. the pipeline fill and `graph_iters` iterations of the method are each
-//      captured once into a CUDA graph (all scalars live in the device control
-//      block, so the same graphs are valid for every restart and iteration);
-//   2. fill graph, then iteration-graph launches, two in flight, with the
-//      status words copied back asynchronously after each; iterations after
-//      convergence are no-ops;
+//   1. the pipeline fill is launched kernel by kernel; meanwhile the host records
+//      two iterations into a CUDA graph (all scalars live in the device control
+//      block, so a graph is valid for every iteration and restart), launches it
+//      for the first `graph_iters` iterations, and records the graph of
+//      `graph_iters` iterations while the GPU works on those.  Recording and
+//      instantiating the long graph before the first launch left the GPU idle
+//      for 0.5 ms of every solve (64^3 PIPEGCR: 706 us for a solve of no
+//      iterations); launching the first iterations kernel by kernel costs ~7 us
+//      per kernel against ~4 us in a graph;
+//   2. iteration-graph launches, two batches in flight, with the status words
+//      copied back asynchronously after each; iterations after convergence are
+//      no-ops, and no batch is launched past maxit;
 //   3. on convergence the true residual ||b - A x|| is checked (residual
 //      replacement: restart from x with a tightened target when it fails); on a
 //      norm breakdown the method restarts from x, flushing the pipeline
@@ -97,8 +103,10 @@ struct Graph {
   }
 };
 
+// Records what `body` enqueues on cs; instantiates it unless only the number of
+// its kernels is wanted.
 template <typename F>
-cudaError_t capture(cudaStream_t cs, Graph& out, F&& body) {
+cudaError_t capture(cudaStream_t cs, Graph& out, bool instantiate, F&& body) {
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
   cudaError_t eb = body();
@@ -113,7 +121,7 @@ cudaError_t capture(cudaStream_t cs, Graph& out, F&& body) {
     cudaGraphNodeType t;
     if (cudaGraphNodeGetType(n, &t) == cudaSuccess && t == cudaGraphNodeTypeKernel) out.kernels++;
   }
-  return cudaGraphInstantiate(&out.x, out.g, 0);
+  return instantiate ? cudaGraphInstantiate(&out.x, out.g, 0) : cudaSuccess;
 }
 
 struct Events {
@@ -212,13 +220,13 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
 
   long long kernel_launches = 0;
 
-  // ---- ||b|| ----
-  double bnorm = 0.0;
+  SolveCtl* hc = ctx->pinned;   // pinned status copies (owned by the context)
+  double* h_bb = reinterpret_cast<double*>(hc + 2);   // pinned: <b, b>, <b - A x, b - A x>
+
+  // ---- ||b||: read after the first synchronisation below ----
   PFK_CUDA(ctx, dot_into(ctx, b, b, N, d_out, st));
   kernel_launches += 1;
-  PFK_CUDA(ctx, cudaMemcpyAsync(&bnorm, d_out, sizeof(double), cudaMemcpyDeviceToHost, st));
-  PFK_CUDA(ctx, cudaStreamSynchronize(st));
-  bnorm = std::sqrt(bnorm);
+  PFK_CUDA(ctx, cudaMemcpyAsync(h_bb, d_out, sizeof(double), cudaMemcpyDeviceToHost, st));
   double sigma_used = NAN;
   PFK_CUDA(ctx, M->prepare(env, b, d_out, &sigma_used));
   const bool gmres = M->cycle_length() > 0;
@@ -229,41 +237,42 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
   const bool profile = prm->profile != 0;
   Events pev;
   if (profile) PFK_CUDA(ctx, pev.make(2 * K, cudaEventDefault));
-  Graph gfill, giter;
-  {
-    SolveEnv cenv = env;
-    cenv.st = ctx->cap_stream;
-    cudaError_t e = capture(cenv.st, gfill, [&]() -> cudaError_t {
-      ctl_restart_kernel<<<1, 1, 0, cenv.st>>>(ctl);
-      cudaError_t e2 = cudaGetLastError();
-      if (e2 != cudaSuccess) return e2;
-      return M->fill(cenv, b, x);
-    });
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "capture pipeline fill");
-    e = capture(cenv.st, giter, [&]() -> cudaError_t {
+  constexpr int kShort = 2;
+  Graph gfill, giter, gshort;   // (gfill: only counted)
+  SolveEnv cenv = env;
+  cenv.st = ctx->cap_stream;
+  auto record = [&](Graph& g, int iters, bool instantiate) -> cudaError_t {
+    return capture(cenv.st, g, instantiate, [&]() -> cudaError_t {
       cudaError_t e2 = cudaSuccess;
-      for (int g = 0; g < K && e2 == cudaSuccess; ++g) {
+      for (int q = 0; q < iters && e2 == cudaSuccess; ++q) {
         SolveEnv ienv = cenv;
         if (profile) {
-          ienv.pass_ev0 = pev.v[2 * g];
-          ienv.pass_ev1 = pev.v[2 * g + 1];
+          ienv.pass_ev0 = pev.v[2 * q];
+          ienv.pass_ev1 = pev.v[2 * q + 1];
         }
         e2 = M->iteration(ienv, x);
       }
       return e2;
     });
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "capture iteration");
-  }
+  };
+  auto fill = [&](const SolveEnv& fenv) -> cudaError_t {
+    ctl_restart_kernel<<<1, 1, 0, fenv.st>>>(ctl);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : M->fill(fenv, b, x);
+  };
 
-  SolveCtl* hc = ctx->pinned;   // pinned status copies (owned by the context)
   Events ev, tev;
   PFK_CUDA(ctx, ev.make(2, cudaEventDisableTiming));
   PFK_CUDA(ctx, tev.make(2, cudaEventDefault));
 
   PFK_CUDA(ctx, cudaEventRecord(tev.v[0], st));
 
-  const double goal = std::fmax(prm->rtol * bnorm, prm->atol);
+  double bnorm = NAN, goal = NAN;
   int restarts = 0, breakdowns = 0, replacements = 0;
+  SolveCtl cur = h;             // the control block as last read
+  int it_known = 0;             // its iterations
+  const int short_iters = M->iterations_per_step() > 1 || K < kShort ? 1 : kShort;
+  int fills = 0;
   bool prev_breakdown = false;
   pfk_status result = PFK_OK;
   double rnorm_true = NAN;
@@ -277,10 +286,10 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
     e = dot_into(ctx, scratch, scratch, N, d_out, st);
     if (e != cudaSuccess) return e;
     kernel_launches += 2;
-    e = cudaMemcpyAsync(out, d_out, sizeof(double), cudaMemcpyDeviceToHost, st);
+    e = cudaMemcpyAsync(h_bb + 1, d_out, sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return e;
     e = cudaStreamSynchronize(st);
-    *out = std::sqrt(*out);
+    *out = std::sqrt(h_bb[1]);
     return e;
   };
   // With profiling, one graph is in flight: after it completes, the event pairs
@@ -297,34 +306,62 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
 
   for (;;) {
     // ---- (re)start: pipeline fill ----
-    PFK_CUDA(ctx, cudaGraphLaunch(gfill.x, st));
-    kernel_launches += gfill.kernels;
-    PFK_CUDA(ctx, cudaMemcpyAsync(&hc[0], ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, st));
-    PFK_CUDA(ctx, cudaStreamSynchronize(st));
-    int status = hc[0].status;
-    if (std::isnan(target)) target = hc[0].target;
-
-    if (status == kRun) {
-      if (hc[0].it >= prm->maxit) {
-        status = kMaxit;
-      } else if (!profile) {
-        // ---- iterate: graph launches, two in flight ----
-        int q = 0;
-        PFK_CUDA(ctx, cudaGraphLaunch(giter.x, st));
-        kernel_launches += giter.kernels;
-        PFK_CUDA(ctx, cudaMemcpyAsync(&hc[q], ctl, sizeof(int) * 4, cudaMemcpyDeviceToHost, st));
-        PFK_CUDA(ctx, cudaEventRecord(ev.v[q], st));
-        for (;;) {
-          PFK_CUDA(ctx, cudaGraphLaunch(giter.x, st));
-          kernel_launches += giter.kernels;
-          PFK_CUDA(ctx, cudaMemcpyAsync(&hc[q ^ 1], ctl, sizeof(int) * 4, cudaMemcpyDeviceToHost, st));
-          PFK_CUDA(ctx, cudaEventRecord(ev.v[q ^ 1], st));
-          PFK_CUDA(ctx, cudaEventSynchronize(ev.v[q]));
-          if (hc[q].status != kRun) break;
-          q ^= 1;
+    PFK_CUDA(ctx, fill(env));
+    int status = kRun;
+    // iterations launched after this fill, counted from the last known total
+    // (a GMRES fill forms a column, which counts too)
+    int64_t reach = it_known;
+    if (!profile && it_known < prm->maxit) {
+      auto launch = [&](int slot) -> cudaError_t {
+        // a batch: the long graph, or short ones up to K iterations or maxit
+        const bool whole = giter.x && prm->maxit - reach >= (int64_t)K * M->iterations_per_step();
+        const Graph& g = whole ? giter : gshort;
+        const int step = whole ? K : short_iters;
+        cudaError_t e = cudaSuccess;
+        for (int q = 0; q < K && e == cudaSuccess && (q == 0 || reach < prm->maxit); q += step) {
+          e = cudaGraphLaunch(g.x, st);
+          kernel_launches += g.kernels;
+          reach += (int64_t)step * M->iterations_per_step();
         }
-      } else {
-        int before = hc[0].passes;
+        if (e != cudaSuccess) return e;
+        e = cudaMemcpyAsync(&hc[slot], ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, st);
+        return e != cudaSuccess ? e : cudaEventRecord(ev.v[slot], st);
+      };
+      int q = 0;
+      const bool first = !gshort.x;
+      if (first) PFK_CUDA(ctx, record(gshort, short_iters, true));
+      PFK_CUDA(ctx, launch(q));
+      if (first) {   // while the GPU works: the fill's kernel count, and the long graph if more is to come
+        PFK_CUDA(ctx, capture(cenv.st, gfill, false, [&]() -> cudaError_t { return fill(cenv); }));
+        if (prm->maxit - reach >= (int64_t)K * M->iterations_per_step()) PFK_CUDA(ctx, record(giter, K, true));
+      }
+      for (;;) {
+        const bool next = reach < prm->maxit;
+        if (next) PFK_CUDA(ctx, launch(q ^ 1));
+        PFK_CUDA(ctx, cudaEventSynchronize(ev.v[q]));
+        if (hc[q].status != kRun) break;
+        if (!next) {
+          reach = hc[q].it;
+          if (reach >= prm->maxit) break;
+          PFK_CUDA(ctx, launch(q ^ 1));
+        }
+        q ^= 1;
+      }
+      // (a batch in flight behind this one changes nothing: its kernels see the status)
+      std::memcpy(&cur, &hc[q], sizeof(SolveCtl));
+    } else {
+      PFK_CUDA(ctx, cudaMemcpyAsync(&hc[0], ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, st));
+      PFK_CUDA(ctx, cudaStreamSynchronize(st));
+      if (!gfill.g) {
+        PFK_CUDA(ctx, capture(cenv.st, gfill, false, [&]() -> cudaError_t { return fill(cenv); }));
+        if (profile) PFK_CUDA(ctx, record(giter, K, true));
+      }
+      std::memcpy(&cur, &hc[0], sizeof(SolveCtl));
+      status = cur.status;
+      if (status == kRun && cur.it >= prm->maxit) {
+        status = kMaxit;
+      } else if (status == kRun) {
+        int before = cur.passes;
         for (;;) {
           PFK_CUDA(ctx, cudaGraphLaunch(giter.x, st));
           kernel_launches += giter.kernels;
@@ -334,11 +371,19 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
           before = hc[1].passes;
           if (hc[1].status != kRun) break;
         }
+        std::memcpy(&cur, &hc[1], sizeof(SolveCtl));
+        status = kRun;
       }
-      PFK_CUDA(ctx, cudaMemcpyAsync(&hc[0], ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, st));
-      PFK_CUDA(ctx, cudaStreamSynchronize(st));
-      if (status == kRun) status = hc[0].status;
     }
+    fills += 1;
+    it_known = cur.it;
+    if (std::isnan(bnorm)) {
+      bnorm = std::sqrt(*h_bb);
+      goal = std::fmax(prm->rtol * bnorm, prm->atol);
+      target = cur.target;
+    }
+    if (status == kRun) status = cur.status;
+    if (status == kRun && cur.it >= prm->maxit) status = kMaxit;   // a fill stopped short of its first iteration
     // GMRES types: least-squares solve over the cycle's valid columns and
     // x = x_0 + U y, whatever ended the cycle
     if (gmres && status != kNonFinite) {
@@ -372,7 +417,7 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
     }
     if (status == kBreakdown) {
       breakdowns += 1;
-      const int i_since = hc[0].i;
+      const int i_since = cur.i;
       if ((i_since <= 1 && prev_breakdown) || restarts >= prm->max_restarts) {
         set_error(ctx, "norm breakdown persisted after restarting");
         result = PFK_ERR_BREAKDOWN;
@@ -406,17 +451,17 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
     result = PFK_ERR_CUDA;
     break;
   }
+  kernel_launches += (long long)fills * gfill.kernels;
   PFK_CUDA(ctx, cudaEventRecord(tev.v[1], st));
   if (result != PFK_OK || std::isnan(rnorm_true)) {
     double rt = 0.0;
     PFK_CUDA(ctx, true_residual(&rt));
     rnorm_true = rt;
   }
-  PFK_CUDA(ctx, cudaMemcpyAsync(&hc[0], ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, st));
   PFK_CUDA(ctx, cudaStreamSynchronize(st));
   float ms = 0.f;
   PFK_CUDA(ctx, cudaEventElapsedTime(&ms, tev.v[0], tev.v[1]));
-  const int hl = hc[0].hist_len;
+  const int hl = cur.hist_len;
   if (prm->history && hist_cap > 0) {
     const int ncopy = hl < hist_cap ? hl : hist_cap;
     if (ncopy > 0)
@@ -425,20 +470,20 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
   }
   if (info) {
     info->status = result;
-    info->iterations = hc[0].it;
+    info->iterations = cur.it;
     info->restarts = restarts;
     info->breakdowns = breakdowns;
     info->replacements = replacements;
     info->history_len = hl;
-    info->rho0 = hc[0].rho0;
-    info->rho_final = hc[0].rho;
+    info->rho0 = cur.rho0;
+    info->rho_final = cur.rho;
     info->rnorm_true = rnorm_true;
     info->bnorm = bnorm;
     info->time_ms = ms;
-    info->pass_launches = hc[0].passes;
+    info->pass_launches = cur.passes;
     info->kernel_launches = (int32_t)(kernel_launches > INT32_MAX ? INT32_MAX : kernel_launches);
-    info->pass_bytes = hc[0].alg_bytes;
-    info->pass_flops = hc[0].alg_flops;
+    info->pass_bytes = cur.alg_bytes;
+    info->pass_flops = cur.alg_flops;
     info->pass_ms = profile ? pass_ms : 0.0;
   }
   return result;

@@ -47,6 +47,8 @@ class Method {
   // Called by the driver when an iteration group stopped with status kRun at
   // the end of a restart cycle (GMRES types); default: nothing.
   virtual cudaError_t end_cycle(const SolveEnv& env, double* x) { (void)env; (void)x; return cudaSuccess; }
+  // Iterations one call of iteration() covers at most.
+  virtual int iterations_per_step() const { return 1; }
   // Number of ring/Hessenberg columns (GMRES types restart after this many).
   virtual int cycle_length() const { return 0; }
   // Once per solve, before bind: picks the persistent single-launch form when
