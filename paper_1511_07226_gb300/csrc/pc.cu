@@ -500,6 +500,9 @@ static StencilT<V, C> make_stencil(const pfk_operator* op, const C* d, const C* 
 template <typename V, typename C>
 static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v, double* out, const double* add,
                              const int* status, cudaStream_t st) {
+  if constexpr (std::is_same<V, double>::value) {
+    if (pcg_resident_fits(pc)) return pcg_resident(pc, v, out, add, status, st);
+  }
   const int64_t n = A.n;
   V* base = (V*)pc->buf;
   V* r = base;
@@ -836,6 +839,7 @@ extern "C" pfk_status pfk_pc_apply_inner_pcg_noalloc(pfk_context* ctx, const pfk
   tmp.kind = PFK_PC_INNER_PCG;
   tmp.inner = inner_iters;
   tmp.precision = PFK_FP64;
+  tmp.separate = true;
   tmp.buf = scratch;
   tmp.buf_bytes = 5 * (size_t)op->n * sizeof(double);
   tmp.partials = scratch + 5 * kNoallocMaxN;

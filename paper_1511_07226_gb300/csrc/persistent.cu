@@ -116,11 +116,16 @@ __device__ __forceinline__ bool grid_barrier(SolveCtl* ctl) {
       ctl->bar_count = 0u;
       red_add_release(&ctl->bar_gen, 1u);
     } else {
-      const unsigned long long t0 = global_ns();
+      // polls of one word; the abort word and the timer are read on every 16th
+      // (with them on every poll a release was noticed up to 2 us late)
+      unsigned long long t0 = 0ull;
       const long long budget = ctl->bar_timeout_ns;
-      while (ld_acquire(&ctl->bar_gen) == g) {
+      for (unsigned polls = 0; ld_acquire(&ctl->bar_gen) == g; ++polls) {
+        if (budget > 0 && (polls & 15u)) continue;
         if (ld_acquire(&ctl->bar_abort)) { ok = 0; break; }
-        if (budget <= 0 || global_ns() - t0 > (unsigned long long)budget) {
+        const unsigned long long t = global_ns();
+        if (t0 == 0ull) t0 = t;
+        if (budget <= 0 || t - t0 > (unsigned long long)budget) {
           atomicExch(&ctl->bar_abort, 1u);
           ok = 0;
           break;

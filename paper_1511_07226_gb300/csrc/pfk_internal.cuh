@@ -87,6 +87,10 @@ struct PcCtl {
   long long calls;         // noisy preconditioner: applications so far
   double scale;            // noisy preconditioner: eta ||v|| / ||xi_j|| of the current application
   long long row;           // noisy preconditioner: j mod count of the current application
+  unsigned int bar_count;  // grid barrier of the resident inner PCG: arrivals,
+  unsigned int bar_gen;    // generation,
+  unsigned int bar_abort;  // set when a wait timed out
+  unsigned int bar_pad;
 };
 
 }  // namespace pfk
@@ -164,6 +168,8 @@ struct pfk_pc {
   pfk::PcCtl* ctl = nullptr;
   double* partials = nullptr;
   int partials_cap = 0;         // doubles in `partials` (bounds the grid of the reduction kernels)
+  bool separate = false;        // inner PCG as separate kernels at every size (the allocation-free entry
+                                // point: a cooperative launch may allocate, and its scratch is shared)
   // noisy preconditioner: the noise bank (count x n) and 1 / ||xi_j||
   double noise_eta = 0.0;
   double* bank = nullptr;
@@ -460,6 +466,11 @@ cudaError_t op_apply(const pfk_operator* op, const double* x, double* y, const d
 // out = add + B(v) (add may be null).  `status` as above.
 cudaError_t pc_apply(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,
                      cudaStream_t st);
+
+// FP64 inner PCG in one cooperative launch (pcg_resident.cu).
+bool pcg_resident_fits(const pfk_pc* pc);
+cudaError_t pcg_resident(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,
+                         cudaStream_t st);
 
 // Nested block preconditioner (nested.cu).
 cudaError_t nested_apply(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,
