@@ -71,22 +71,45 @@ class Method {
 // Window dots, the reduction of the CR types and the base methods: one
 // register accumulator per window slot and thread (independent FMAs, the
 // loads of a whole window in flight), then warp_sum_transposed.  acc[j] +=
-// <v, s_j> over the elements e = first, first + step, ...; s_off holds the
-// slots' offsets.  body(e, v_e) adds the caller's own products.
+// <v, s_j>; s_off holds the slots' offsets.  body(e, v_e) adds the caller's own
+// products.  The loop is instantiated for window sizes rounded up to 4: with
+// one loop for 32 slots the guarded products of the empty slots were issued all
+// the same (101x97x93: 79 us at every window size).
 constexpr int kWinThreads = 128;
-constexpr int kWinBlocksPerSm = 5;   // 93 registers at NW = 32
+constexpr int kWinBlocksPerSm = 4;   // 128 registers: no spills at 32 slots
+
+template <int NR, int NW, typename F>
+__device__ __forceinline__ void window_dots_loop(const double* __restrict__ v, const double* __restrict__ S,
+                                                 const size_t* s_off, int nu, int64_t N, double (&acc)[NW],
+                                                 F&& body) {
+  for (int64_t e = (int64_t)blockIdx.x * kWinThreads + threadIdx.x; e < N; e += (int64_t)gridDim.x * kWinThreads) {
+    const double ve = __ldg(&v[e]);
+#pragma unroll
+    for (int j = 0; j < NR; ++j) {
+      // rows below NR - 3 exist; the last ones may not
+      const double sv = (j < NR - 3 || j < nu) ? __ldg(&S[s_off[j] + e]) : 0.0;
+      acc[j] = fma(ve, sv, acc[j]);
+    }
+    body(e, ve);
+  }
+}
 
 template <int NW, typename F>
 __device__ __forceinline__ void window_dots(const double* __restrict__ v, const double* __restrict__ S,
                                             const size_t* s_off, int nu, int64_t N, double (&acc)[NW], F&& body) {
 #pragma unroll
   for (int j = 0; j < NW; ++j) acc[j] = 0.0;
-  for (int64_t e = (int64_t)blockIdx.x * kWinThreads + threadIdx.x; e < N; e += (int64_t)gridDim.x * kWinThreads) {
-    const double ve = __ldg(&v[e]);
-#pragma unroll
-    for (int j = 0; j < NW; ++j)
-      if (j < nu) acc[j] = fma(ve, __ldg(&S[s_off[j] + e]), acc[j]);
-    body(e, ve);
+  if (nu <= 4) window_dots_loop<4>(v, S, s_off, nu, N, acc, body);
+  else if (nu <= 8) window_dots_loop<8>(v, S, s_off, nu, N, acc, body);
+  else if constexpr (NW >= 16) {
+    if (nu <= 12) window_dots_loop<12>(v, S, s_off, nu, N, acc, body);
+    else if (nu <= 16) window_dots_loop<16>(v, S, s_off, nu, N, acc, body);
+    else if constexpr (NW >= 32) {
+      if (nu <= 20) window_dots_loop<20>(v, S, s_off, nu, N, acc, body);
+      else if (nu <= 24) window_dots_loop<24>(v, S, s_off, nu, N, acc, body);
+      else if (nu <= 28) window_dots_loop<28>(v, S, s_off, nu, N, acc, body);
+      else window_dots_loop<32>(v, S, s_off, nu, N, acc, body);
+    }
   }
 }
 
