@@ -8,6 +8,7 @@
 #include "pfk_internal.cuh"
 #include "solver.cuh"
 #include "stencil.cuh"
+#include "stencil_flat.cuh"
 
 #include <cmath>
 
@@ -268,6 +269,32 @@ __global__ void __launch_bounds__(kTileThreads) base_apply_dots_walk(TiledStenci
   base_apply_scalars<MODE>(ctl, i, slots, s_sum[0], s_sum[1], s_sum[2]);
 }
 
+// The same on the flat rows (ncu, 101x97x93, FCG's eta: 44.8 -> 20.4 us, of which the
+// dots no longer formed are a third).
+template <bool ADV, int MODE>
+__global__ void __launch_bounds__(kThreads) base_apply_dots_flat(FlatStencil A, double* __restrict__ P,
+                                                                 double* __restrict__ S, const double* __restrict__ r,
+                                                                 int64_t N, SolveCtl* ctl, double* partials) {
+  if (ctl->status != kRun) return;
+  constexpr int ND = ApplyDots<MODE>::nd;
+  const bool fill = (MODE == kApplyFcgFill || MODE == kApplyGcrFill);
+  const int i = fill ? 0 : ctl->i + 1;
+  const int slots = ctl->mmax + 1;
+  const size_t off = (size_t)(i % slots) * (size_t)N;
+  BaseApplyEpi<MODE> e{S + off, r, {}};
+  const double* p = P + off;
+  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
+    const auto pre = e.pre(c);
+    double pv;
+    const double sv = flat_row<ADV>(A, p, c, pv);
+    e(c, sv, pv, pre);
+  }
+  __shared__ double s_sum[3];
+  if (!reduce_last_block_fast<ND>(e.acc, partials, &ctl->counter, s_sum)) return;
+  if (threadIdx.x != 0) return;
+  base_apply_scalars<MODE>(ctl, i, slots, s_sum[0], s_sum[1], s_sum[2]);
+}
+
 static int base_template(int mmax) { return mmax <= 8 ? 8 : mmax <= 16 ? 16 : 32; }
 
 static cudaError_t launch_window_dots(const SolveEnv& env, int tmpl, const double* v, const double* r,
@@ -296,6 +323,15 @@ template <int MODE>
 static cudaError_t launch_apply_dots(const SolveEnv& env, double* P, double* S, const double* r) {
   const pfk_operator* op = env.op;
   constexpr int ND = ApplyDots<MODE>::nd;
+  if (!op->rowptr && flat_stencil_fits(op)) {
+    const FlatStencil F = flat_stencil(op);
+    const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
+    const int blocks = stream_blocks(env.ctx, env.N, 4);
+    if (!env.partials_fit(blocks, ND)) return cudaErrorInvalidValue;
+    if (adv) base_apply_dots_flat<true, MODE><<<blocks, kThreads, 0, env.st>>>(F, P, S, r, env.N, env.ctl, env.partials);
+    else base_apply_dots_flat<false, MODE><<<blocks, kThreads, 0, env.st>>>(F, P, S, r, env.N, env.ctl, env.partials);
+    return cudaGetLastError();
+  }
   if (!op->rowptr) {
     TiledStencil<double, double> T;
     const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
@@ -500,10 +536,30 @@ __global__ void __launch_bounds__(kTileThreads) fgb_apply_store_walk(TiledStenci
   tiled_stencil_walk<double, double, ADV, 1>(T, ucur, e);
 }
 
+template <bool ADV>
+__global__ void __launch_bounds__(kThreads) fgb_apply_store_flat(FlatStencil A, const double* __restrict__ ucur,
+                                                                 double* __restrict__ U, double* __restrict__ z,
+                                                                 int64_t N, const FgState* gs, const int* status) {
+  if (*status != kRun) return;
+  double* u = U + (size_t)gs->k * (size_t)N;
+  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
+    double uv;
+    z[c] = flat_row<ADV>(A, ucur, c, uv);
+    u[c] = uv;
+  }
+}
+
 static cudaError_t launch_apply_store(const SolveEnv& env, const double* ucur, double* U, double* z,
                                       const FgState* gs, const int* status) {
   const pfk_operator* op = env.op;
-  if (!op->rowptr) {
+  if (!op->rowptr && flat_stencil_fits(op)) {
+    const FlatStencil F = flat_stencil(op);
+    const int blocks = stream_blocks(env.ctx, env.N, 8);
+    if (op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0)
+      fgb_apply_store_flat<true><<<blocks, kThreads, 0, env.st>>>(F, ucur, U, z, env.N, gs, status);
+    else
+      fgb_apply_store_flat<false><<<blocks, kThreads, 0, env.st>>>(F, ucur, U, z, env.N, gs, status);
+  } else if (!op->rowptr) {
     TiledStencil<double, double> T;
     const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
     const int slots = adv ? tiled_stencil_slots(fgb_apply_store_walk<true>, env.ctx->num_sms)

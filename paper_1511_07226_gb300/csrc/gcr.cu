@@ -23,6 +23,7 @@
 #include "pfk_internal.cuh"
 #include "solver.cuh"
 #include "stencil.cuh"
+#include "stencil_flat.cuh"
 
 namespace pfk {
 
@@ -240,6 +241,27 @@ __global__ void __launch_bounds__(kTileThreads) pipegcr_apply_walk(TiledStencil<
   }
 }
 
+// The same on the flat rows (64^3: 12.8 -> 8.7 us).
+template <bool ADV>
+__global__ void __launch_bounds__(kThreads) pipegcr_apply_flat(FlatStencil A, GcrArgs a) {
+  SolveCtl* ctl = a.ctl;
+  if (ctl->status != kRun) return;
+  GcrApplyEpi e{a.w, a.t, a.r, 0.0, 0.0, 0.0};
+  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
+    const auto pre = e.pre(c);
+    double uc;
+    const double wv = flat_row<ADV>(A, a.u, c, uc);
+    e(c, wv, uc, pre);
+  }
+  double acc[3] = {e.g0, e.g1, e.g2};
+  __shared__ double sums[3];
+  if (reduce_last_block_fast<3>(acc, a.partials, &ctl->counter, sums) && threadIdx.x == 0) {
+    ctl->pend[0] = sums[0];
+    ctl->pend[1] = sums[1];
+    ctl->pend[2] = sums[2];
+  }
+}
+
 // <w_i, s_k> over the window (window_dots); the last block adds the
 // walk's gamma, delta, ||r||^2 and runs the scalar phase of iteration i.
 template <int NW>
@@ -360,7 +382,12 @@ class PipeGcr : public Method {
         case 16: pipegcr_advance<16><<<ablocks, kThreads, 0, env.st>>>(a); break;
         default: pipegcr_advance<32><<<ablocks, kThreads, 0, env.st>>>(a); break;
       }
-      if (adv) pipegcr_apply_walk<true><<<wblocks, kTileThreads, 0, env.st>>>(T, a);
+      if (flat_stencil_fits(op)) {
+        const FlatStencil F = flat_stencil(op);
+        if (!env.partials_fit(ablocks, 3)) return cudaErrorInvalidValue;
+        if (adv) pipegcr_apply_flat<true><<<ablocks, kThreads, 0, env.st>>>(F, a);
+        else pipegcr_apply_flat<false><<<ablocks, kThreads, 0, env.st>>>(F, a);
+      } else if (adv) pipegcr_apply_walk<true><<<wblocks, kTileThreads, 0, env.st>>>(T, a);
       else pipegcr_apply_walk<false><<<wblocks, kTileThreads, 0, env.st>>>(T, a);
       const int sf = adv ? 10 : 7;
       switch (tmpl) {

@@ -7,6 +7,7 @@
 // "A" of every listing (Algs. 2-15).
 #include "pfk_internal.cuh"
 #include "stencil.cuh"
+#include "stencil_flat.cuh"
 
 #include <cmath>
 #include <cstring>
@@ -159,6 +160,20 @@ __global__ void __launch_bounds__(kTileThreads) stencil_tiled_apply_kernel(Tiled
   tiled_stencil_walk<double, double, ADV, 1>(A, m, e);
 }
 
+// The same on the flat form.
+template <bool ADV>
+__global__ void __launch_bounds__(kThreads) stencil_flat_apply_kernel(FlatStencil A, const double* __restrict__ m,
+                                                                      double* __restrict__ y,
+                                                                      const double* __restrict__ bsub,
+                                                                      const int* __restrict__ status) {
+  if (status && *status != kRun) return;
+  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
+    double mc;
+    const double v = flat_row<ADV>(A, m, c, mc);
+    y[c] = bsub ? bsub[c] - v : v;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // CSR
 // ---------------------------------------------------------------------------
@@ -255,6 +270,12 @@ cudaError_t op_apply(const pfk_operator* op, const double* x, double* y, const d
   const int blocks = stream_blocks(op->ctx, op->n, 8);
   if (op->rowptr) {
     csr_apply_kernel<<<blocks, kThreads, 0, st>>>(op->rowptr, op->colidx, op->vals, x, y, bsub, op->n, status);
+  } else if (flat_stencil_fits(op)) {
+    const FlatStencil A = flat_stencil(op);
+    if (op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0)
+      stencil_flat_apply_kernel<true><<<blocks, kThreads, 0, st>>>(A, x, y, bsub, status);
+    else
+      stencil_flat_apply_kernel<false><<<blocks, kThreads, 0, st>>>(A, x, y, bsub, status);
   } else {
     TiledStencil<double, double> A;
     const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
