@@ -195,67 +195,18 @@ __device__ __forceinline__ void cgcr_fill_scalars(SolveCtl* ctl, double gamma, d
 // w for Alg. 11).  Convergence test first (as in the listings' order), then
 // beta_{i,k} = -c_k / eta_k, eta_i = delta_i - sum_k beta_{i,k}^2 eta_k (k
 // ascending), alpha_i = gamma_i / eta_i; eta_i <= 0 is a norm breakdown.
-__device__ __forceinline__ void cgcr_iteration_scalars(SolveCtl* ctl, int i, int nu, double gamma, double delta,
-                                                       double rr, const double* c) {
-  const int slots = ctl->mmax + 1;
-  ctl->it += 1;
-  ctl->i = i;
-  ctl->gamma = gamma;
-  ctl->delta = delta;
-  const double rnorm = sqrt(rr);
-  const double rho = cgcr_rho(ctl, gamma, rr);
-  ctl->rho = rho;
-  const int hslot = ctl->hist_len;
-  push_history(ctl, rho, rnorm, nan(""), nan(""));
-  if (!isfinite(rho)) { ctl->status = kNonFinite; return; }
-  if (rho <= ctl->target) { ctl->status = kConverged; return; }
-  double sumb = 0.0;
-  for (int jj = 0; jj < nu; ++jj) {
-    const int k = i - nu + jj;
-    const double ek = ctl->eta_ring[k % slots];
-    const double b = -c[jj] / ek;
-    ctl->beta[jj] = b;
-    sumb += b * b * ek;
-  }
-  const double eta = delta - sumb;
-  const double al = eta != 0.0 ? gamma / eta : nan("");
-  ctl->eta = eta;
-  ctl->alpha = al;
-  ctl->nw = nu;
-  ctl->eta_ring[i % slots] = eta;
-  if (ctl->history && hslot < ctl->hist_cap) {
-    ctl->history[(size_t)hslot * PFK_HISTORY_FIELDS + 2] = eta;
-    ctl->history[(size_t)hslot * PFK_HISTORY_FIELDS + 3] = al;
-  }
-  if (eta <= 0.0) { ctl->status = kBreakdown; return; }
-  if (ctl->it >= ctl->maxit) { ctl->status = kMaxit; return; }
-}
-
-// cgcr_iteration_scalars by all threads of the (last) block: the nu window
-// betas -c_k / eta_k (each a global load of eta_k and a division) are formed
-// in parallel, one per thread, and thread 0 accumulates eta_i in the same k
-// order; everything else is thread 0's, in the same statement order.  c is
-// the window's dots in k order (shared or global memory); s_tmp holds 2 * cap
-// + 1 doubles of shared memory, cap >= nu.
+//
+// Run by all threads of the (last) block (at least 96): the nu betas (each a
+// global load of eta_k and a division) one per thread of warp 0, rho and the
+// convergence test by thread 32 and ||r_i|| by thread 64 meanwhile -- a division
+// or square root is a chain of FP64 instructions of about a microsecond --, then
+// thread 0 accumulates eta_i.  The betas of an iteration that stops here are
+// not used.  c: shared or global memory; s_tmp holds 2 * cap + 1 doubles of
+// shared memory, cap >= nu.
 __device__ __forceinline__ void cgcr_iteration_scalars_block(SolveCtl* ctl, int i, int nu, double gamma, double delta,
                                                              double rr, const double* c, double* s_tmp, int cap) {
+  __shared__ double s_rho, s_rnorm;
   int* s_go = (int*)(s_tmp + 2 * cap);
-  if (threadIdx.x == 0) {
-    ctl->it += 1;
-    ctl->i = i;
-    ctl->gamma = gamma;
-    ctl->delta = delta;
-    const double rnorm = sqrt(rr);
-    const double rho = cgcr_rho(ctl, gamma, rr);
-    ctl->rho = rho;
-    s_go[1] = ctl->hist_len;
-    push_history(ctl, rho, rnorm, nan(""), nan(""));
-    s_go[0] = 1;
-    if (!isfinite(rho)) { ctl->status = kNonFinite; s_go[0] = 0; }
-    else if (rho <= ctl->target) { ctl->status = kConverged; s_go[0] = 0; }
-  }
-  __syncthreads();
-  if (!s_go[0]) return;
   const int slots = ctl->mmax + 1;
   if ((int)threadIdx.x < nu) {
     const int k = i - nu + (int)threadIdx.x;
@@ -264,24 +215,38 @@ __device__ __forceinline__ void cgcr_iteration_scalars_block(SolveCtl* ctl, int 
     ctl->beta[threadIdx.x] = b;
     s_tmp[threadIdx.x] = b * b;
     s_tmp[cap + threadIdx.x] = ek;
+  } else if (threadIdx.x == 32) {
+    const double rho = cgcr_rho(ctl, gamma, rr);
+    s_rho = rho;
+    ctl->rho = rho;
+    s_go[0] = 1;
+    if (!isfinite(rho)) { ctl->status = kNonFinite; s_go[0] = 0; }
+    else if (rho <= ctl->target) { ctl->status = kConverged; s_go[0] = 0; }
+  } else if (threadIdx.x == 64) {
+    s_rnorm = sqrt(rr);
   }
   __syncthreads();
   if (threadIdx.x != 0) return;
+  const int it = ctl->it + 1;
+  ctl->it = it;
+  ctl->i = i;
+  ctl->gamma = gamma;
+  ctl->delta = delta;
+  if (!s_go[0]) {
+    push_history(ctl, s_rho, s_rnorm, nan(""), nan(""));
+    return;
+  }
   double sumb = 0.0;
   for (int jj = 0; jj < nu; ++jj) sumb = fma(s_tmp[jj], s_tmp[cap + jj], sumb);
   const double eta = delta - sumb;
   const double al = eta != 0.0 ? gamma / eta : nan("");
-  const int hslot = s_go[1];
   ctl->eta = eta;
   ctl->alpha = al;
   ctl->nw = nu;
   ctl->eta_ring[i % slots] = eta;
-  if (ctl->history && hslot < ctl->hist_cap) {
-    ctl->history[(size_t)hslot * PFK_HISTORY_FIELDS + 2] = eta;
-    ctl->history[(size_t)hslot * PFK_HISTORY_FIELDS + 3] = al;
-  }
+  push_history(ctl, s_rho, s_rnorm, eta, al);
   if (eta <= 0.0) { ctl->status = kBreakdown; return; }
-  if (ctl->it >= ctl->maxit) { ctl->status = kMaxit; return; }
+  if (it >= ctl->maxit) { ctl->status = kMaxit; return; }
 }
 
 }  // namespace pfk
