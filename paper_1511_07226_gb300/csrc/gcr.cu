@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kTileThreads) pipegcr_apply_walk(TiledStencil<
   }
 }
 
-// The same on the flat rows (64^3: 12.8 -> 8.7 us).
+// The same on the flat rows (64^3, whole tiles: the same time; ragged sides gain as in ops.cu).
 template <bool ADV>
 __global__ void __launch_bounds__(kThreads) pipegcr_apply_flat(FlatStencil A, GcrArgs a) {
   SolveCtl* ctl = a.ctl;

@@ -38,6 +38,7 @@
 #include "group.cuh"
 #include "pfk_internal.cuh"
 #include "solver.cuh"
+#include "stencil_flat.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -112,6 +113,8 @@ struct GrpSys {
   int u0, u1, u2;
   int adv;            // any advection weight non-zero
   int nblk;           // CTAs of the group
+  int sx, sy;         // c / nx = (c mx) >> sx, row / ny = (row my) >> sy for c < 2^31 (mx = 0: larger system)
+  unsigned mx, my;
   int pad0;
   const double* b;
   double* x;
@@ -252,6 +255,30 @@ __device__ void grp_sum(const GrpSys& S, GrpCta* g, const double (&v)[ND], doubl
          i += 32)                                                                                    \
       for (int64_t c = row_ * (S).nx + i, once_ = 1; once_; once_ = 0)
 
+// f(c, i, j, k) for the CTA's cells.  FLAT: 32 consecutive cells per warp,
+// whatever the row length -- an FP64 instruction holds the pipe as long with a
+// few active lanes as with 32, and a row per warp leaves 24 of 64 lanes idle at
+// nx = 40.  Otherwise a row per warp (the order the FP32 inner products were
+// pinned with, and systems of 2^31 cells or more).
+template <bool FLAT, typename F>
+__device__ __forceinline__ void grp_cells(const GrpSys& S, const GrpCta* g, F&& f) {
+  if (FLAT && S.mx) {
+    const unsigned nx = (unsigned)S.nx, ny = (unsigned)S.ny;
+    const unsigned end = (unsigned)(g->row_hi * S.nx);
+    const unsigned beg = (unsigned)(g->row_lo * S.nx);
+#pragma unroll 2
+    for (unsigned q = beg + threadIdx.x; q < end; q += kGrpThreads) {
+      const unsigned c = beg + (end - 1u - q);   // from the end: what the loop before wrote last is read first
+      const unsigned row = (unsigned)(((unsigned long long)c * S.mx) >> S.sx);
+      const unsigned k = (unsigned)(((unsigned long long)row * S.my) >> S.sy);
+      f((int64_t)c, (int)(c - row * nx), (int)(row - k * ny), (int)k);
+    }
+  } else {
+#pragma unroll 2
+    GRP_ROWS(S, g, c, i, j, k) f(c, i, j, k);
+  }
+}
+
 // The operator's coefficients in the arithmetic type V of a kernel phase: the
 // FP64 arrays, or the FP32 copies of the FP32 inner preconditioner.
 template <typename V>
@@ -309,13 +336,23 @@ __device__ __forceinline__ double grp_row(const GrpSys& S, const double* m, int6
 // every CTA of the group (the caller passed a system barrier since it was
 // last written).
 __device__ void grp_apply(const GrpSys& S, GrpCta* g, const double* m, double* y, const double* bsub) {
-  #pragma unroll 2
-  GRP_ROWS(S, g, c, i, j, k) {
+  grp_cells<true>(S, g, [&](int64_t c, int i, int j, int k) {
     const double v = grp_row(S, m, c, i, j, k);
     y[c] = bsub ? bsub[c] - v : v;
-  }
+  });
   __syncthreads();
 }
+
+// FP32 -> FP64 by integer operations: the hardware conversion runs on the FP64
+// pipe (about 64 cycles per warp instruction, as much as the product it feeds).
+// Zeros, subnormals, infinities and NaN take the conversion instruction.
+__device__ __forceinline__ double grp_d(float v) {
+  const unsigned b = __float_as_uint(v);
+  if ((b & 0x7f800000u) - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+  return (double)v;
+}
+__device__ __forceinline__ double grp_d(double v) { return v; }
 
 // Inner Jacobi-PCG in V (FP64, or FP32 vectors and coefficient copies with
 // the inner products of FP32 values accumulated in FP64): out = add + x_k.
@@ -329,6 +366,9 @@ __device__ void grp_pcg(const GrpSys& S, GrpCta* g, const GrpCoef<V>& A, const d
   V* x = s + n;
   const V* dinv = A.dinv;
   const int kk = S.P.pc_inner;
+  // FP64: D^-1 r, which gamma needs, is kept (as p_0, later in s in place of
+  // s_{i-1}) and read back by the p update: one product and one load less
+  constexpr bool F64 = sizeof(V) == 8;
   {
     // r_0 = v; gamma_0 = <D^-1 r_0, r_0>
     double acc[1] = {0.0};
@@ -337,7 +377,8 @@ __device__ void grp_pcg(const GrpSys& S, GrpCta* g, const GrpCoef<V>& A, const d
       const V rv = (V)v[e];
       r[e] = rv;
       const V z = dinv[e] * rv;
-      acc[0] += (double)z * (double)rv;
+      if (F64) p[e] = z;
+      acc[0] += grp_d(z) * grp_d(rv);
     }
     grp_sum<1>(S, g, acc, s_red);
     if (threadIdx.x == 0) {
@@ -348,16 +389,17 @@ __device__ void grp_pcg(const GrpSys& S, GrpCta* g, const GrpCoef<V>& A, const d
   }
   if (g->last_x > 0) {
     // p_0 = D^-1 r_0, s_0 = A p_0, eta_0 = <s_0, p_0>
-    #pragma unroll 4
-    GRP_ELEMS(S, g, e) p[e] = dinv[e] * r[e];
-    grp_barrier(S, g);
+    if (!F64) {   // (FP64: formed above; the sum's barrier completed it)
+      #pragma unroll 4
+      GRP_ELEMS(S, g, e) p[e] = dinv[e] * r[e];
+      grp_barrier(S, g);
+    }
     double acc[1] = {0.0};
-    #pragma unroll 2
-    GRP_ROWS(S, g, c, i, j, k) {
+    grp_cells<F64>(S, g, [&](int64_t c, int i, int j, int k) {
       const V sv = grp_row_t<V>(S, A, p, c, i, j, k);
       s[c] = sv;
-      acc[0] += (double)sv * (double)p[c];
-    }
+      acc[0] += grp_d(sv) * grp_d(p[c]);
+    });
     grp_sum<1>(S, g, acc, s_red);
     if (threadIdx.x == 0) {
       if (g->red[0] == 0.0) g->last_x = 0;
@@ -376,7 +418,8 @@ __device__ void grp_pcg(const GrpSys& S, GrpCta* g, const GrpCoef<V>& A, const d
         const V rv = r[e] - al * s[e];
         r[e] = rv;
         const V z = dinv[e] * rv;
-        acc[0] += (double)z * (double)rv;
+        if (F64) s[e] = z;
+        acc[0] += grp_d(z) * grp_d(rv);
       }
       grp_sum<1>(S, g, acc, s_red);
       if (threadIdx.x == 0) {
@@ -399,7 +442,7 @@ __device__ void grp_pcg(const GrpSys& S, GrpCta* g, const GrpCoef<V>& A, const d
       GRP_ELEMS(S, g, e) {
         const V po = p[e];
         x[e] = (it == 1 ? V(0) : x[e]) + al * po;
-        if (do_p) p[e] = dinv[e] * r[e] + be * po;
+        if (do_p) p[e] = F64 ? s[e] + be * po : dinv[e] * r[e] + be * po;
       }
       if (!do_p) {
         __syncthreads();
@@ -410,12 +453,11 @@ __device__ void grp_pcg(const GrpSys& S, GrpCta* g, const GrpCoef<V>& A, const d
     {
       // s_i = A p_i, eta_i
       double acc[1] = {0.0};
-      #pragma unroll 2
-      GRP_ROWS(S, g, c, i, j, k) {
+      grp_cells<F64>(S, g, [&](int64_t c, int i, int j, int k) {
         const V sv = grp_row_t<V>(S, A, p, c, i, j, k);
         s[c] = sv;
-        acc[0] += (double)sv * (double)p[c];
-      }
+        acc[0] += grp_d(sv) * grp_d(p[c]);
+      });
       grp_sum<1>(S, g, acc, s_red);
       if (threadIdx.x == 0) {
         if (g->red[0] == 0.0) g->last_x = it;
@@ -430,8 +472,8 @@ __device__ void grp_pcg(const GrpSys& S, GrpCta* g, const GrpCoef<V>& A, const d
   GRP_ELEMS(S, g, e) {
     double y;
     if (last_x == 0) y = 0.0;
-    else if (kk <= last_x) y = (double)((kk == 1 ? V(0) : x[e]) + al * p[e]);
-    else y = (double)x[e];
+    else if (kk <= last_x) y = grp_d((kk == 1 ? V(0) : x[e]) + al * p[e]);
+    else y = grp_d(x[e]);
     out[e] = add ? add[e] + y : y;
   }
   grp_barrier(S, g);
@@ -723,12 +765,11 @@ __device__ void grp_gcr_dots(const GrpSys& S, GrpCta* g, double* smem) {
   const double* Sr = S.ws + 7 * n + (int64_t)slots * n;
   const int i = st->i + 1;
   const int nu = nu_window(i, S.P.mmax, S.P.truncation);
-  #pragma unroll 2
-  GRP_ROWS(S, g, c, ii, j, k) {
+  grp_cells<true>(S, g, [&](int64_t c, int ii, int j, int k) {
     const double wv = grp_row(S, vu, c, ii, j, k);
     vw[c] = wv;
     vt[c] = wv - vr[c];
-  }
+  });
   if (threadIdx.x < nu) g->s_off[threadIdx.x] = (size_t)((i - nu + (int)threadIdx.x) % slots) * (size_t)n;
   __syncthreads();
   double* s_sk = smem;
@@ -1457,6 +1498,12 @@ pfk_status GroupRunner::admit(const pfk_operator* op, const pfk_pc_desc* pcd, co
   S.u0 = op->upw[0]; S.u1 = op->upw[1]; S.u2 = op->upw[2];
   S.adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
   S.nblk = nblk;
+  S.mx = S.my = 0u;
+  S.sx = S.sy = 0;
+  if (flat_stencil_fits(op)) {
+    const FlatStencil F = flat_stencil(op);
+    S.mx = F.mx; S.my = F.my; S.sx = F.sx; S.sy = F.sy;
+  }
   S.b = b_dev;
   S.x = x_dev;
   S.ws = (double*)mem;
