@@ -36,7 +36,11 @@
 // global memory, the partial rows fetched with asynchronous 16-byte copies.
 // On this GPU an FP64 instruction costs its sub-partition tens of
 // nanoseconds whatever its active lanes, so the reductions and the scalar
-// phase are arranged to keep such instructions few and off one warp's chain.
+// phase are arranged to keep such instructions few and off one warp's chain
+// (48 iterations of 64 x 64 with host arrays: 842 -> 793 us, 12.3 us an
+// iteration with windows up to 30, by the exchange-step sums, one direction
+// per thread of a row, more row groups in sum_partials and three scalar chains
+// side by side).
 // Block 0 keeps the control block up to date (status, counters, history) for
 // the host driver.
 #include "pfk_internal.cuh"
@@ -105,8 +109,10 @@ __device__ __forceinline__ void red_add_release(unsigned int* p, unsigned int v)
 // others wait for it with acquire loads.  The wait is bounded (the control
 // block's bar_timeout_ns, 2 s by default): on time-out the block raises
 // bar_abort, and a raised bar_abort ends every other wait.
-// Returns false in that case.
-__device__ __forceinline__ bool grid_barrier(SolveCtl* ctl) {
+// Returns false in that case.  meanwhile() runs in the other threads while
+// thread 0 waits.
+template <typename F>
+__device__ __forceinline__ bool grid_barrier(SolveCtl* ctl, F&& meanwhile) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -133,9 +139,15 @@ __device__ __forceinline__ bool grid_barrier(SolveCtl* ctl) {
       }
     }
     s_ok = ok;
+  } else {
+    meanwhile();
   }
   __syncthreads();
   return s_ok != 0;
+}
+
+__device__ __forceinline__ bool grid_barrier(SolveCtl* ctl) {
+  return grid_barrier(ctl, [] {});
 }
 
 // Sum of a value over the eight rows a warp holds, for the thread position q
@@ -170,12 +182,22 @@ __device__ __forceinline__ void wait_partials() {
 // order into out[j] (shared memory).  Each FP64 instruction costs a
 // sub-partition tens of nanoseconds whatever its lane count, so the work is
 // spread over (column, row group) tasks that keep all lanes busy: task t of
-// the block sums rows g, g + G, g + 2G, ... of column j (t = g * nd + j, G =
-// the groups that fit in the block's threads, at most 4), then thread j adds
-// the G group sums in group order.  Every block gets bitwise the same sums.
-__device__ __forceinline__ void sum_partials(const double* s_part, int nb, int nd, double* out, double* s_grp) {
+// the block sums rows g, g + G, g + 2G, ... of column j (t = g * nd + j), then
+// thread j adds the G group sums in group order: nb / G + G additions in a
+// row.  G is as many groups as fit in the block's threads, at most gmax =
+// sqrt(nb), beyond which the second sum grows by more than the first shrinks
+// (nb = 128, 16 columns: 24 additions, where at most 4 groups took 36).  Every
+// block gets bitwise the same sums.
+__device__ __forceinline__ int max_groups(int nb) {
+  int G = 1;
+  while ((G + 1) * (G + 1) <= nb) ++G;
+  return G;
+}
+
+__device__ __forceinline__ void sum_partials(const double* s_part, int nb, int nd, int gmax, double* out,
+                                             double* s_grp) {
   int G = kPerThreads / nd;
-  G = G < 1 ? 1 : (G > 4 ? 4 : G);
+  G = G < 1 ? 1 : (G > gmax ? gmax : G);
   for (int t = threadIdx.x; t < G * nd; t += kPerThreads) {
     const int g = t / nd, j = t - g * nd;
     double a = 0.0;
@@ -195,27 +217,40 @@ __device__ __forceinline__ void sum_partials(const double* s_part, int nb, int n
 // threads' values.  Thread q of a row holds scalar column q in scq (its own
 // product, computed from the row's values every thread of the row has) and
 // window columns 4 s + q in acc[s].  Layout: [scalar 0..3, window 0 .. nw-1].
-// Each column is summed over the warp's rows by three shuffle steps (lanes of
-// equal q), then over the four warps in order.
+// The columns are summed over the warp's eight rows by three exchange steps in
+// which a lane hands over half of the columns it still holds, so NWQ - 1 (+ 3 -
+// log2 NWQ) additions sum NWQ columns a lane, not the 3 NWQ of as many shuffle
+// trees (the same additions, 7 for 24 at NWQ = 8: 0.6 us of a pass's chain),
+// then over the four warps in order.
 template <int NWQ>
-__device__ __forceinline__ void write_pipefcg_row(double scq, const double (&acc)[NWQ], int nw, double* s_red,
-                                                  double* row) {
+__device__ __forceinline__ void write_pipefcg_row(double scq, double (&acc)[NWQ], int nw, double* s_red, double* row) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & 3;
   {
     const double v = quad_col_sum(scq);
     if (lane < 4) s_red[warp * kPerNd + q] = v;
   }
+  int s = 0, m = 4;
 #pragma unroll
-  for (int s = 0; s < NWQ; ++s) {
-    const double v = quad_col_sum(acc[s]);
+  for (int h = NWQ / 2; h > 0; h >>= 1, m <<= 1) {
+    const bool up = (lane & m) != 0;
+#pragma unroll
+    for (int j = 0; j < h; ++j) {
+      const double keep = up ? acc[j + h] : acc[j], send = up ? acc[j] : acc[j + h];
+      acc[j] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+    }
+    if (up) s += h;
+  }
+#pragma unroll
+  for (int o = 4 * NWQ; o < 32; o <<= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+  {
     const int j = 4 * s + q;
-    if (lane < 4 && j < nw) s_red[warp * kPerNd + 4 + j] = v;
+    if (lane < 4 * NWQ && j < nw) s_red[warp * kPerNd + 4 + j] = acc[0];
   }
   __syncthreads();
   for (int j = threadIdx.x; j < 4 + nw; j += blockDim.x) {
-    double v = 0.0;
+    double v = s_red[j];
 #pragma unroll
-    for (int w = 0; w < kPerThreads / 32; ++w) v += s_red[w * kPerNd + j];
+    for (int w = 1; w < kPerThreads / 32; ++w) v += s_red[w * kPerNd + j];
     row[j] = v;
   }
 }
@@ -227,11 +262,12 @@ struct PerState {
   int truncation, norm, maxit, hist_cap;   // copies of the control block's constants
   double target;
   double* history;
-  int passes;                              // work counters of this launch (block 0 adds them at the end)
-  double alg_bytes, alg_flops;
+  int passes;                              // iterations of this launch and the sum of their windows: the
+  long long windows;                       // work counters are formed from them at its end, by block 0
   double alpha, gamma, delta, eta, rho;
   double beta[PFK_MAX_MMAX];
   double eta_ring[PFK_MAX_MMAX + 1];
+  double inv_eta[PFK_MAX_MMAX + 1];        // 1 / eta_ring (PIPEFCG)
   double sums[kPerNd];
   double cw[PFK_MAX_MMAX + 1];
   double tmp[2 * PFK_MAX_MMAX + 2];
@@ -256,11 +292,13 @@ __device__ __forceinline__ void load_state(PerState* st, const SolveCtl* ctl) {
     st->target = ctl->target;
     st->history = ctl->history;
     st->passes = 0;
-    st->alg_bytes = 0.0;
-    st->alg_flops = 0.0;
+    st->windows = 0;
   }
   for (int j = threadIdx.x; j < PFK_MAX_MMAX; j += blockDim.x) st->beta[j] = ctl->beta[j];
-  for (int j = threadIdx.x; j <= PFK_MAX_MMAX; j += blockDim.x) st->eta_ring[j] = ctl->eta_ring[j];
+  for (int j = threadIdx.x; j <= PFK_MAX_MMAX; j += blockDim.x) {
+    st->eta_ring[j] = ctl->eta_ring[j];
+    st->inv_eta[j] = 1.0 / st->eta_ring[j];   // of a slot in use; the others are not read
+  }
   __syncthreads();
 }
 
@@ -294,11 +332,15 @@ __device__ __forceinline__ void store_state(const PerState* st, SolveCtl* ctl, i
 }
 
 // Block 0 adds the launch's work counters to the control block (at exit).
-__device__ __forceinline__ void store_counters(const PerState* st, SolveCtl* ctl) {
+// Words of a pass per row: u, w, m, n, x, r, D^-1 and 4 nu history read; p, s,
+// q, z, x, r, u, w, m written.  FP64 flops: 4 nu MAXPY, 4 advance and nu + 4
+// dot FMAs, the Jacobi product and two additions.
+__device__ __forceinline__ void store_counters(const PerState* st, SolveCtl* ctl, int64_t N) {
   if (blockIdx.x != 0 || threadIdx.x != 0 || st->passes == 0) return;
+  const double np = (double)st->passes, nw = (double)st->windows;
   ctl->passes += st->passes;
-  ctl->alg_bytes += st->alg_bytes;
-  ctl->alg_flops += st->alg_flops;
+  ctl->alg_bytes += 8.0 * (double)N * (4.0 * nw + 16.0 * np);
+  ctl->alg_flops += (double)N * (2.0 * (5.0 * nw + 8.0 * np) + 3.0 * np);
 }
 
 // ---------------------------------------------------------------------------
@@ -446,7 +488,7 @@ __host__ __device__ __forceinline__ PerLayout per_layout(int64_t N, int nb, int 
 // ---------------------------------------------------------------------------
 
 template <int NW>
-__global__ void __launch_bounds__(kPerThreads) pipefcg_persistent(PersistArgs a) {
+__global__ void __launch_bounds__(kPerThreads, 1) pipefcg_persistent(PersistArgs a) {
   constexpr int NWQ = NW / 4;
   extern __shared__ __align__(16) double s_dyn[];
   __shared__ PerState st;
@@ -484,7 +526,10 @@ __global__ void __launch_bounds__(kPerThreads) pipefcg_persistent(PersistArgs a)
   double* sm = R.vec(4);
   double* sn = R.vec(5);
   const double* sd = R.vec(6);
+  const double* dfrom = q == 0 ? su : q == 1 ? sw : q == 2 ? sm : sn;   // thread q's direction update starts from this,
+  double* vown = q == 0 ? sx : q == 1 ? sr : q == 2 ? su : sw;          // and the vector it advances
   const bool jacobi = a.dinv != nullptr;
+  const int gmax = max_groups(nb);
 
   for (int g = 0; g < a.iters; ++g) {
     if (st.status != kRun) break;
@@ -522,50 +567,48 @@ __global__ void __launch_bounds__(kPerThreads) pipefcg_persistent(PersistArgs a)
           skv[s] = sv;
         }
       }
-      sp += __shfl_xor_sync(0xffffffffu, sp, 1);
-      ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-      sq += __shfl_xor_sync(0xffffffffu, sq, 1);
-      sz += __shfl_xor_sync(0xffffffffu, sz, 1);
-      sp += __shfl_xor_sync(0xffffffffu, sp, 2);
-      ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-      sq += __shfl_xor_sync(0xffffffffu, sq, 2);
-      sz += __shfl_xor_sync(0xffffffffu, sz, 2);
-      double un = 0.0, p = 0.0, s = 0.0, qv = 0.0, z = 0.0, xn = 0.0, rn = 0.0, wn = 0.0, mn = 0.0;
+      // Thread q of the row goes on with sum q only: the window sums over the
+      // row's four threads by two exchange steps (3 additions, not the 8 of
+      // four shuffle trees; the same sums), then dir = p, s, q, z for q = 0..3
+      // (u, w, m, n + its sum) and nv = x, r, u, w advanced with it.
+      const bool up1 = (q & 1) != 0, up2 = (q & 2) != 0;
+      const double lo = (up1 ? ss : sp) + __shfl_xor_sync(0xffffffffu, up1 ? sp : ss, 1);
+      const double hi = (up1 ? sz : sq) + __shfl_xor_sync(0xffffffffu, up1 ? sq : sz, 1);
+      const double win = (up2 ? hi : lo) + __shfl_xor_sync(0xffffffffu, up2 ? lo : hi, 2);
+      double dir = 0.0, nv = 0.0;
       if (valid) {
-        const double u0 = su[l], w0 = sw[l];
-        p = u0 + sp;
-        s = w0 + ss;
-        qv = sm[l] + sq;
-        z = sn[l] + sz;
-        xn = fma(alpha, p, sx[l]);
-        rn = fma(-alpha, s, sr[l]);
-        un = fma(-alpha, qv, u0);
-        wn = fma(-alpha, z, w0);
+        dir = dfrom[l] + win;
+        nv = fma(q == 0 ? alpha : -alpha, dir, vown[l]);
+      }
+      const double s = __shfl_sync(0xffffffffu, dir, 1, 4), rn = __shfl_sync(0xffffffffu, nv, 1, 4);
+      const double un = __shfl_sync(0xffffffffu, nv, 2, 4), wn = __shfl_sync(0xffffffffu, nv, 3, 4);
+      double mn = 0.0;
+      if (valid) {
         const double t = wn - rn;                            // B's input w_i - r_i (eq. BwMinusR)
         const double y = jacobi ? __dmul_rn(sd[l], t) : t;
         mn = __dadd_rn(un, y);                               // m_i = u_i + B(w_i - r_i)
         const double lf = q == 2 ? rn : un, rt = q == 0 ? rn : q == 1 ? wn : q == 2 ? rn : s;
         scq = fma(lf, rt, scq);
       }
-      __syncwarp();   // every lane of the row has read the old values before thread 0 of the row writes
-      if (valid && q == 0) {
-        R.ring(0, cslot)[l] = p;
-        R.ring(1, cslot)[l] = s;
-        R.ring(2, cslot)[l] = qv;
-        R.ring(3, cslot)[l] = z;
-        sx[l] = xn;
-        sr[l] = rn;
-        su[l] = un;
-        sw[l] = wn;
-        sm[l] = mn;
-        mnew[e] = mn;
+      __syncwarp();   // every lane of the row has read the old values before any of them writes
+      if (valid) {
+        R.ring(q, cslot)[l] = dir;
+        vown[l] = nv;
+        if (q == 0) {
+          sm[l] = mn;
+          mnew[e] = mn;
+        }
       }
 #pragma unroll
-      for (int s2 = 0; s2 < NWQ; ++s2) acc[s2] = fma(un, skv[s2], acc[s2]);
+      for (int s2 = 0; s2 < NWQ; ++s2)
+        if (4 * s2 < nwp) acc[s2] = fma(un, skv[s2], acc[s2]);
     }
     write_pipefcg_row<NWQ>(scq, acc, nwp, s_red, part + (size_t)blockIdx.x * kPerNd);
 
-    if (!grid_barrier(ctl)) {
+    const bool met = grid_barrier(ctl, [&] {
+      if (threadIdx.x == 96) st.inv_eta[cslot] = 1.0 / st.eta_ring[cslot];   // for the scalar phase
+    });
+    if (!met) {
       if (blockIdx.x == 0 && threadIdx.x == 0) ctl->status = kTimeout;
       return;
     }
@@ -579,12 +622,16 @@ __global__ void __launch_bounds__(kPerThreads) pipefcg_persistent(PersistArgs a)
       if (e >= 0 && q == 0) sn[l] = csr_row(a, cs, mnew, e, l);
     }
     wait_partials();
-    sum_partials(s_part, nb, 4 + nwp, st.sums, s_red);
+    sum_partials(s_part, nb, 4 + nwp, gmax, st.sums, s_red);
 
     // ---- scalar phase of iteration i (Alg. 8), the same in every block ----
-    // Warp 1 (thread 32) forms rho_i and the convergence verdict and writes the
-    // history while warp 0 forms the betas, eta_i and alpha_i (used only when
-    // the iteration goes on): the two chains run on different sub-partitions.
+    // Three chains side by side, on different sub-partitions (what the last two
+    // form is used only when the iteration goes on): thread 32 forms rho_i and
+    // the convergence verdict and writes the history; warp 2 forms the betas;
+    // warp 0 forms eta_i and alpha_i without waiting for them, from beta^2
+    // eta_k = (c / eta_k) c with the reciprocals kept beside eta_k (a division
+    // is a chain of some ten FP64 instructions; one rounding more than c /
+    // eta_k, one less than beta * beta * eta_k).
     const int nu = nu_window(i, a.mmax, st.truncation);
     if (threadIdx.x == 32) {
       const double gamma = st.sums[0], rr = st.sums[2];
@@ -593,17 +640,25 @@ __global__ void __launch_bounds__(kPerThreads) pipefcg_persistent(PersistArgs a)
       per_push_history(&st, ctl, rho, st.history ? sqrt(rr) : nan(""), nan(""), nan(""));
       st.go = !isfinite(rho) ? -1 : (rho <= st.target ? 0 : 1);
     }
+    // window dots in order k = i-1-nwp .. i-1 (W_{i-1}, then s_{i-1}); W_i is the last nu
+    const auto window_dot = [&](int jj) {
+      const int c = nwp + 1 - nu + jj;
+      return c < nwp ? st.sums[4 + c] : st.sums[3];
+    };
+    if (threadIdx.x >= 64 && (int)threadIdx.x < 64 + nu) {
+      const int jj = (int)threadIdx.x - 64;
+      st.beta[jj] = -window_dot(jj) / st.eta_ring[(i - nu + jj) % slots];
+    }
     if (threadIdx.x < 32) {
-      // window dots in order k = i-1-nwp .. i-1 (W_{i-1}, then s_{i-1}); W_i is the last nu
       const int jj = (int)threadIdx.x;
       double term = 0.0;
       if (jj < nu) {
-        const int c = nwp + 1 - nu + jj;
-        const double cv = c < nwp ? st.sums[4 + c] : st.sums[3];
-        const double ek = st.eta_ring[(i - nu + jj) % slots];
-        const double bb = -cv / ek;
-        st.beta[jj] = bb;
-        term = (bb * bb) * ek;
+        const double cv = window_dot(jj);
+        const int ks = (i - nu + jj) % slots;
+        const double ek = st.eta_ring[ks];
+        // a reciprocal near the ends of the exponent range is not used
+        const unsigned ex = ((unsigned)__double2hiint(ek) >> 20) & 0x7ffu;
+        term = (ex - 23u < 2000u ? cv * st.inv_eta[ks] : cv / ek) * cv;
       }
       // sum of beta^2 eta over the window: a fixed shuffle tree
       term = warp_sum(term);
@@ -617,6 +672,8 @@ __global__ void __launch_bounds__(kPerThreads) pipefcg_persistent(PersistArgs a)
     if (threadIdx.x == 0) {
       st.it += 1;
       st.i = i;
+      st.passes += 1;
+      st.windows += nwp;
       st.gamma = st.sums[0];
       st.delta = st.sums[1];
       if (st.go < 0) { st.status = kNonFinite; st.go = 0; }
@@ -633,14 +690,6 @@ __global__ void __launch_bounds__(kPerThreads) pipefcg_persistent(PersistArgs a)
       }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      st.passes += 1;
-      // pass words per row: u, w, m, n, x, r, D^-1 and 4 nu history read; p, s,
-      // q, z, x, r, u, w, m written.  FP64 flops: 4 nu MAXPY, 4 advance and
-      // nu + 4 dot FMAs, the Jacobi product and two additions.
-      st.alg_bytes += 8.0 * (double)N * (double)(4 * nwp + 16);
-      st.alg_flops += (double)N * (2.0 * (5 * nwp + 8) + 3.0);
-    }
     store_state(&st, ctl, st.go ? nu : 0, slots);
     __syncthreads();
   }
@@ -650,7 +699,7 @@ __global__ void __launch_bounds__(kPerThreads) pipefcg_persistent(PersistArgs a)
     double* gr[4] = {a.P, a.S, a.Q, a.Z};
     resident_copy(R, gv, gr, 4, nb, N, false);
   }
-  store_counters(&st, ctl);
+  store_counters(&st, ctl, N);
 }
 
 // ---------------------------------------------------------------------------
@@ -658,7 +707,7 @@ __global__ void __launch_bounds__(kPerThreads) pipefcg_persistent(PersistArgs a)
 // ---------------------------------------------------------------------------
 
 template <int NW>
-__global__ void __launch_bounds__(kPerThreads) fcg_persistent(PersistArgs a) {
+__global__ void __launch_bounds__(kPerThreads, 1) fcg_persistent(PersistArgs a) {
   constexpr int NWQ = NW / 4;
   extern __shared__ __align__(16) double s_dyn[];
   __shared__ PerState st;
@@ -695,6 +744,7 @@ __global__ void __launch_bounds__(kPerThreads) fcg_persistent(PersistArgs a) {
   double* su = R.vec(2);
   const double* sd = R.vec(3);
   const bool jacobi = a.dinv != nullptr;
+  const int gmax = max_groups(nb);
 
   for (int g = 0; g < a.iters; ++g) {
     if (st.status != kRun) break;
@@ -737,7 +787,7 @@ __global__ void __launch_bounds__(kPerThreads) fcg_persistent(PersistArgs a) {
     }
     fetch_partials(red1, nb, s_part);
     wait_partials();
-    sum_partials(s_part, nb, 4 + nu, st.sums, s_red);
+    sum_partials(s_part, nb, 4 + nu, gmax, st.sums, s_red);
     // Alg. 2: gamma_i, convergence (thread 32), beta_{i,k} = -<u_i, s_k> / eta_k
     // (warp 0, used only when the iteration goes on)
     if (threadIdx.x == 32) {
@@ -810,7 +860,7 @@ __global__ void __launch_bounds__(kPerThreads) fcg_persistent(PersistArgs a) {
     }
     fetch_partials(red3, nb, s_part);
     wait_partials();
-    sum_partials(s_part, nb, 1, st.sums, s_red);
+    sum_partials(s_part, nb, 1, gmax, st.sums, s_red);
     if (threadIdx.x == 0) {
       // Alg. 2: eta_i = <p_i, s_i>, alpha_i = gamma_i / eta_i
       const double eta = st.sums[0];

@@ -106,3 +106,23 @@ def test_window_dots_sizes(ctx, method, mmax):
     x, info, hist = pfk.solve(ctx, op, pc, b, method=method, mmax=mmax, rtol=1e-14, maxit=its, history=64)
     assert info["iterations"] == ref.iterations
     assert np.linalg.norm(x - ref.x) <= 1e-10 * np.linalg.norm(ref.x)
+
+
+@pytest.mark.parametrize("exponent", [-510, -490, 490, 505])
+def test_single_launch_pipefcg_extreme_scales(ctx, exponent):
+    """eta_k ~ scale^2 outside the range whose reciprocals are kept (2^-1000 ..
+    2^1000), against the one-kernel-per-step path at the same scale (its dots
+    meet the same subnormal products): a few units of 2^-53 per iteration,
+    amplified by 8 iterations at contrast 1e3 by less than 1e4:
+    8 x 4 x 1.1e-16 x 1e4 < 1e-10."""
+    from paper_1511_07226_gb300 import pfk
+    c = W.poisson2d_inclusions()
+    op = pfk.Operator.stencil(ctx, c["dims"], c["eta"], storage="csr")
+    pc = pfk.Preconditioner(ctx, op, "jacobi")
+    kw = dict(method="pipefcg", mmax=30, rtol=1e-14, maxit=8)
+    b = np.ldexp(np.asarray(c["b"], dtype=np.float64), exponent)
+    x0, i0, _ = pfk.solve(ctx, op, pc, b, persistent="off", **kw)
+    x1, i1, _ = pfk.solve(ctx, op, pc, b, persistent="on", **kw)
+    assert i0["iterations"] == i1["iterations"] == 8
+    x0, x1 = np.ldexp(x0, -exponent), np.ldexp(x1, -exponent)
+    assert np.linalg.norm(x1 - x0) <= 1e-10 * np.linalg.norm(x0)
