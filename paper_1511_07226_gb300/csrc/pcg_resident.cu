@@ -15,6 +15,16 @@
 // in the same order, so all hold bitwise the same scalars.  The statements per
 // cell are those of the separate kernels.
 //
+// A barrier and the sum behind it take 3 to 4 us, in which the warps that do
+// not wait have nothing to do, so work that depends on neither is placed there:
+// the x update during the sum for gamma, and the x and y terms of the stencil
+// while p becomes complete everywhere (64^3, four inner iterations: 90.5 ->
+// 88 -> 85 us; 101 x 97 x 93: 146 -> 140 us).  The registers are kept to two
+// blocks per SM although a launch has one, so that the applications of two
+// solves on different streams run side by side: with all registers for one
+// block 64^3 takes 83 us, but a burst of small solves on several workers 29 ms
+// instead of 21.
+//
 // Every wait is bounded (2 s): a wait that runs out raises an abort word that
 // ends all other waits, and the output is set to NaN.
 #include "pfk_internal.cuh"
@@ -98,9 +108,12 @@ struct ResShared {
 };
 
 // Grid barrier; false when a wait gave up (all threads of the block agree).
-__device__ __forceinline__ bool res_barrier(const ResArgs& a, ResShared& sh) {
+// meanwhile(t, nt), t < nt, runs in the other warps while warp 0 waits.
+template <typename G>
+__device__ __forceinline__ bool res_barrier(const ResArgs& a, ResShared& sh, G&& meanwhile) {
   __syncthreads();
-  if (threadIdx.x == 0) sh.ok = res_arrive_wait(a.ctl, sh.gen++);
+  if (threadIdx.x >= 32) meanwhile((int)threadIdx.x - 32, kResThreads - 32);
+  else if (threadIdx.x == 0) sh.ok = res_arrive_wait(a.ctl, sh.gen++);
   __syncthreads();
   return sh.ok != 0;
 }
@@ -112,9 +125,11 @@ __device__ __forceinline__ bool res_barrier(const ResArgs& a, ResShared& sh) {
 // forms the quotient (a division is a chain of FP64 instructions; in all sixteen
 // warps it held the FP64 pipes for 1.5 us).  parity alternates from one sum to
 // the next, so a block that runs ahead never overwrites a partial sum that
-// another still reads.
-template <typename F>
-__device__ __forceinline__ bool res_sum(const ResArgs& a, ResShared& sh, double acc, int parity, F&& quot) {
+// another still reads.  meanwhile(t, nt), t < nt, runs in the warps of
+// the three sub-partitions that warp 0 is not on, while it waits and combines.
+template <typename F, typename G>
+__device__ __forceinline__ bool res_sum(const ResArgs& a, ResShared& sh, double acc, int parity, F&& quot,
+                                        G&& meanwhile) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   sh.buf[threadIdx.x] = acc;
   __syncthreads();
@@ -145,6 +160,8 @@ __device__ __forceinline__ bool res_sum(const ResArgs& a, ResShared& sh, double 
       sh.quot = quot(s);
       sh.ok = ok;
     }
+  } else if (warp & 3) {
+    meanwhile(((warp >> 2) * 3 + (warp & 3) - 1) * 32 + lane, kResThreads / 4 * 3);
   }
   __syncthreads();
   return sh.ok != 0;
@@ -175,6 +192,30 @@ __global__ void __launch_bounds__(kResThreads, 2) pcg_resident_kernel(ResArgs a)
   bool ok = sh.part[0] == 0.0;
   __syncthreads();
 
+  // Terms of (A p)_q up to the y neighbours, in the walk's order.  They are
+  // formed before the barrier that completes p, while it is waited for, for the
+  // cells whose x and y neighbours lie in the block (all but its first and last
+  // nx cells), and kept in s; the z and advection terms follow after it.
+  auto at = [&](int q, int o) { return (unsigned)(q + o) < (unsigned)cells ? p[q + o] : __ldcg(&a.p[lo + q + o]); };
+  auto xy_terms = [&](int q) {
+    const int c = lo + q;
+    const unsigned f = nb[q];
+    const double mxm = (f & 1u) ? at(q, -1) : 0.0, kxm = (f & 1u) ? a.kx[c - 1] : 0.0;
+    const double mxp = (f & 2u) ? at(q, 1) : 0.0;
+    const double mym = (f & 4u) ? at(q, -nx) : 0.0, kym = (f & 4u) ? a.ky[c - nx] : 0.0;
+    const double myp = (f & 8u) ? at(q, nx) : 0.0;
+    double y = a.d[c] * p[q];
+    y -= kxm * mxm;
+    y -= a.kx[c] * mxp;
+    y -= kym * mym;
+    y -= a.ky[c] * myp;
+    return y;
+  };
+  auto inner_terms = [&](int t, int nt) {
+#pragma unroll 2
+    for (int q = nx + t; q < cells - nx; q += nt) s[q] = xy_terms(q);
+  };
+
   // r_0 = v, p_0 = D^-1 r_0, gamma_0 = <D^-1 r_0, r_0>
   double acc = 0.0;
   for (int q = threadIdx.x; q < cells; q += kResThreads) {
@@ -188,7 +229,7 @@ __global__ void __launch_bounds__(kResThreads, 2) pcg_resident_kernel(ResArgs a)
     a.p[c] = z;
     acc = fma(z, rv, acc);
   }
-  ok = ok && res_sum(a, sh, acc, 0, [](double) { return 0.0; });
+  ok = ok && res_sum(a, sh, acc, 0, [](double) { return 0.0; }, inner_terms);
   double gamma = sh.sum, alpha = 0.0;
   int parity = 1;
   bool last = false;     // the final x still needs alpha p
@@ -200,36 +241,27 @@ __global__ void __launch_bounds__(kResThreads, 2) pcg_resident_kernel(ResArgs a)
       for (int q = threadIdx.x; q < cells; q += kResThreads) {
         const int c = lo + q;
         const unsigned f = nb[q];
-        auto at = [&](int o) { return (unsigned)(q + o) < (unsigned)cells ? p[q + o] : __ldcg(&a.p[c + o]); };
         const double mc = p[q];
-        const double mxm = (f & 1u) ? at(-1) : 0.0, kxm = (f & 1u) ? a.kx[c - 1] : 0.0;
-        const double mxp = (f & 2u) ? at(1) : 0.0;
-        const double mym = (f & 4u) ? at(-nx) : 0.0, kym = (f & 4u) ? a.ky[c - nx] : 0.0;
-        const double myp = (f & 8u) ? at(nx) : 0.0;
         double mzm = 0.0, kzm = 0.0, mzp = 0.0, kzc = 0.0;
         if (a.nz > 1) {
           kzc = a.kz[c];
-          if (f & 16u) { mzm = at(-sxy); kzm = a.kz[c - sxy]; }
-          if (f & 32u) mzp = at(sxy);
+          if (f & 16u) { mzm = at(q, -sxy); kzm = a.kz[c - sxy]; }
+          if (f & 32u) mzp = at(q, sxy);
         }
-        double y = a.d[c] * mc;
-        y -= kxm * mxm;
-        y -= a.kx[c] * mxp;
-        y -= kym * mym;
-        y -= a.ky[c] * myp;
+        double y = q >= nx && q < cells - nx ? s[q] : xy_terms(q);
         if (a.nz > 1) {
           y -= kzm * mzm;
           y -= kzc * mzp;
         }
         if (ADV) {
-          y -= a.a0 * (a.u0 < 0 ? mxm : mxp);
-          y -= a.a1 * (a.u1 < 0 ? mym : myp);
+          y -= a.a0 * ((f & (a.u0 < 0 ? 1u : 2u)) ? at(q, a.u0 < 0 ? -1 : 1) : 0.0);
+          y -= a.a1 * ((f & (a.u1 < 0 ? 4u : 8u)) ? at(q, a.u1 < 0 ? -nx : nx) : 0.0);
           if (a.nz > 1) y -= a.a2 * (a.u2 < 0 ? mzm : mzp);
         }
         s[q] = y;
         acc = fma(y, mc, acc);
       }
-      if (!(ok = res_sum(a, sh, acc, parity, [=](double eta) { return gamma / eta; }))) break;
+      if (!(ok = res_sum(a, sh, acc, parity, [=](double eta) { return gamma / eta; }, [](int, int) {}))) break;
       parity ^= 1;
       if (sh.sum == 0.0) break;      // eta_i
       alpha = sh.quot;
@@ -244,10 +276,14 @@ __global__ void __launch_bounds__(kResThreads, 2) pcg_resident_kernel(ResArgs a)
         const double rv = fma(-alpha, s[q], r[q]), z = a.dinv[lo + q] * rv;
         r[q] = rv;
         s[q] = z;
-        x[q] = fma(alpha, p[q], x[q]);
         acc = fma(z, rv, acc);
       }
-      if (!(ok = res_sum(a, sh, acc, parity, [=](double g) { return g / gamma; }))) break;
+      // nothing waits for x: its update fills the FP64 pipes during the reduction
+      ok = res_sum(a, sh, acc, parity, [=](double g) { return g / gamma; }, [&](int t, int nt) {
+#pragma unroll 4
+        for (int q = t; q < cells; q += nt) x[q] = fma(alpha, p[q], x[q]);
+      });
+      if (!ok) break;
       parity ^= 1;
       if (sh.sum == 0.0) break;      // gamma_{i+1}
       const double beta = sh.quot;
@@ -258,7 +294,7 @@ __global__ void __launch_bounds__(kResThreads, 2) pcg_resident_kernel(ResArgs a)
         p[q] = pv;
         a.p[lo + q] = pv;
       }
-      if (!(ok = res_barrier(a, sh))) break;
+      if (!(ok = res_barrier(a, sh, inner_terms))) break;
     }
   }
   // out = add + x_k
