@@ -270,7 +270,7 @@ pfk_status pfk_pc_apply(pfk_context* ctx, const pfk_pc* pc, const double* v, dou
   CHECK_ARG(ctx, ctx && pc && v && y, "NULL argument");
   CHECK_ARG(ctx, v != y, "v and y must not overlap");
   cudaSetDevice(ctx->device);
-  PFK_CUDA(ctx, pc_apply(pc, v, y, nullptr, nullptr, ctx->stream));
+  PFK_CUDA(ctx, pc_apply(pc, v, y, nullptr, nullptr, ctx->stream, false));
   PFK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   return PFK_OK;
 }

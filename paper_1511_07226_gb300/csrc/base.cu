@@ -89,11 +89,12 @@ __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) base_window_dots
   {
     const double tot = warp_sum_transposed<NW>(acc);
     const int nd = nu + ng;
-    if (lane < nu) s_red[warp * nd + lane] = tot;
+    const int j = lane / (32 / NW);   // the slot whose sum the lane holds
+    if (lane % (32 / NW) == 0 && j < nu) s_red[warp * nd + j] = tot;
     if (ng) {
       double g[2] = {g0, g1};
       const double w = warp_sum_transposed<2>(g);
-      if (lane < 2) s_red[warp * nd + nu + lane] = w;
+      if (lane % 16 == 0) s_red[warp * nd + nu + lane / 16] = w;
     }
     __syncthreads();
   }
@@ -363,6 +364,7 @@ class Fcg : public Method {
     P_ = tmp_ + N; S_ = P_ + (mmax + 1) * N;
   }
   double* scratch() override { return tmp_; }
+  bool blocking() const override { return true; }
   int iterations_per_step() const override { return persistent_ ? kPersistentIters : 1; }
   bool configure(const pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc, int64_t N, int mode) override {
     persistent_ = mode != 1 && persistent_eligible(ctx, op, pc, PFK_FCG, 0, N);
@@ -416,6 +418,7 @@ class Gcr : public Method {
     P_ = tmp_ + N; S_ = P_ + (mmax + 1) * N;
   }
   double* scratch() override { return tmp_; }
+  bool blocking() const override { return true; }
   cudaError_t fill(const SolveEnv& env, const double* b, double* x) override {
     cudaError_t e;
     if ((e = op_apply(env.op, x, r_, b, nullptr, env.st)) != cudaSuccess) return e;   // r_0
@@ -593,7 +596,8 @@ __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) fgb_dots(const d
   double acc[NW];
   window_dots<NW>(z, P, s_off, nk, N, acc, [](int64_t, double) {});
   const double tot = warp_sum_transposed<NW>(acc);
-  if (lane < nk) s_red[warp * nk + lane] = tot;
+  const int j = lane / (32 / NW);   // the slot whose sum the lane holds
+  if (lane % (32 / NW) == 0 && j < nk) s_red[warp * nk + j] = tot;
   __syncthreads();
   if (!combine_block_partials_2l(s_red, nk, partials, ND, &ctl->counter, ctl->gcounter, s_sum)) return;
   if ((int)threadIdx.x < nk) gs->H[threadIdx.x * kGm + gs->k] = s_sum[threadIdx.x];
@@ -705,6 +709,7 @@ class Fgmres : public Method {
     P_ = tmp_ + N; U_ = P_ + (int64_t)(m + 1) * N;
   }
   double* scratch() override { return tmp_; }
+  bool blocking() const override { return true; }
   int cycle_length() const override { return m_; }
   cudaError_t fill(const SolveEnv& env, const double* b, double* x) override {
     const int* status = &env.ctl->status;

@@ -285,7 +285,8 @@ __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) pipegcr_window_d
   double acc[NW];
   window_dots<NW>(a.w, a.S, s_off, nu, N, acc, [](int64_t, double) {});
   const double tot = warp_sum_transposed<NW>(acc);
-  if (lane < nu) s_red[warp * nu + lane] = tot;
+  const int j = lane / (32 / NW);   // the slot whose sum the lane holds
+  if (lane % (32 / NW) == 0 && j < nu) s_red[warp * nu + j] = tot;
   __syncthreads();
   if (!combine_block_partials_2l(s_red, nu, a.partials, NW, &ctl->counter, ctl->gcounter, s_sum)) return;
   if (threadIdx.x == 0) {

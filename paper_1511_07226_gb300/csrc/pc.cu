@@ -535,11 +535,24 @@ static StencilT<V, C> make_stencil(const pfk_operator* op, const C* d, const C* 
   return A;
 }
 
+// Work units of FP64 C_i on the tiled walk: the planes per unit, and with them
+// the order of eta's sum, are chosen for this many resident blocks per SM (what
+// the kernel's 72 registers allow), not for what a later build's registers allow.
+constexpr int kPcgWalkBlocksPerSm = 3;
+
+// FP64, pinned: gamma is summed over a grid of 8 blocks per SM (a thread takes
+// cells c, c + T, ...) and eta over the tiled walk's columns, always: inside a
+// pipelined recurrence another order of these sums changes the iterates far
+// above rounding (128^3, contrast 1e3, 40 iterations: up to 1.6e-8).  Otherwise
+// the faster forms, with sums in their own orders: one launch while the vectors
+// fit in shared memory (64^3, 4 iterations: 133 -> 85 us), else C_i on the flat
+// rows and half the reducing blocks (150 x 141 x 133: 402 -> 378 us).
 template <typename V, typename C>
 static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v, double* out, const double* add,
-                             const int* status, cudaStream_t st) {
-  if constexpr (std::is_same<V, double>::value) {
-    if (pcg_resident_fits(pc)) return pcg_resident(pc, v, out, add, status, st);
+                             const int* status, cudaStream_t st, bool pinned) {
+  constexpr bool F64 = std::is_same<V, double>::value;
+  if constexpr (F64) {
+    if (!pinned && pcg_resident_fits(pc)) return pcg_resident(pc, v, out, add, status, st);
   }
   const int64_t n = A.n;
   V* base = (V*)pc->buf;
@@ -548,16 +561,16 @@ static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v
   V* x = base + 2 * n;
   V* p[2] = {base + 3 * n, base + 4 * n};
   const int k = pc->inner;
-  // reducing kernels: 4 blocks per SM in FP64 (every block adds 12 FP64
-  // instructions to the sum), 8 in FP32, where the FP32 partial sums of a
-  // thread fix the grid
-  const int blocks = stream_blocks(pc->ctx, n, std::is_same<V, double>::value ? 4 : 8);
   const int sblocks = stream_blocks(pc->ctx, n, 8);
+  const int bblocks = F64 ? stream_blocks(pc->ctx, n, 4) : sblocks;   // B_i: two cells per thread and step
+  // reducing kernels: the grid fixes the order of the sums (FP32: a thread's FP32 partial sums)
+  const int blocks = F64 && !pinned ? bblocks : sblocks;
   TiledStencil<V, C> T;
   const pfk_operator* op = pc->op;
   const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
-  const int slots = adv ? tiled_stencil_slots(pcg_c_kernel<V, C, true>, pc->ctx->num_sms)
-                        : tiled_stencil_slots(pcg_c_kernel<V, C, false>, pc->ctx->num_sms);
+  const int slots = F64   ? kPcgWalkBlocksPerSm * pc->ctx->num_sms
+                    : adv ? tiled_stencil_slots(pcg_c_kernel<V, C, true>, pc->ctx->num_sms)
+                          : tiled_stencil_slots(pcg_c_kernel<V, C, false>, pc->ctx->num_sms);
   const int units = tiled_stencil_setup<V, C>(T, op, A.d, A.kx, A.ky, A.kz, slots);
   const int tblocks = units < pc->partials_cap ? units : pc->partials_cap;
   PcCtl* ctl = pc->ctl;
@@ -584,8 +597,8 @@ static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v
         return;
       }
     }
-    if constexpr (std::is_same<V, double>::value) {
-      if (flat_stencil_fits(op)) {
+    if constexpr (F64) {
+      if (!pinned && flat_stencil_fits(op)) {
         const FlatStencil F = flat_stencil(op);
         if (T.adv) pcg_c_flat_kernel<true><<<blocks, kThreads, 0, st>>>(F, pv, s, ctl, i, pc->partials, status);
         else pcg_c_flat_kernel<false><<<blocks, kThreads, 0, st>>>(F, pv, s, ctl, i, pc->partials, status);
@@ -598,8 +611,7 @@ static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v
   pcg_c(p[0], 0);
   for (int i = 1; i < k; ++i) {
     pcg_a_kernel<V, C><<<blocks, kThreads, 0, st>>>(A, v, r, s, ctl, i, pc->partials, status);
-    pcg_b_kernel<V, C><<<blocks, kThreads, 0, st>>>(A, std::is_same<V, double>::value ? s : r, p[(i - 1) & 1],
-                                                    p[i & 1], x, ctl, i, status);
+    pcg_b_kernel<V, C><<<bblocks, kThreads, 0, st>>>(A, F64 ? s : r, p[(i - 1) & 1], p[i & 1], x, ctl, i, status);
     pcg_c(p[i & 1], i);
   }
   pcg_final_kernel<V, C><<<sblocks, kThreads, 0, st>>>(n, p[(k - 1) & 1], x, add, out, ctl, k, status);
@@ -679,7 +691,7 @@ static cudaError_t chebyshev(const pfk_pc* pc, StencilT<V, C> A, const double* v
 }
 
 cudaError_t pc_apply(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,
-                     cudaStream_t st) {
+                     cudaStream_t st, bool pinned) {
   if (pc->kind == PFK_PC_BLOCK_UPPER) return nested_apply(pc, v, out, add, status, st);
   const pfk_operator* op = pc->op;
   const int64_t n = op->n;
@@ -699,13 +711,13 @@ cudaError_t pc_apply(const pfk_pc* pc, const double* v, double* out, const doubl
   if (pc->kind == PFK_PC_INNER_PCG) {
     if (pc->precision == PFK_FP64)
       return inner_pcg<double, double>(pc, make_stencil<double, double>(op, op->d, op->kx, op->ky, op->kz, op->dinv),
-                                       v, out, add, status, st);
+                                       v, out, add, status, st, pinned);
     if (pc->precision == PFK_FP32)
       return inner_pcg<float, float>(pc, make_stencil<float, float>(op, op->d32, op->kx32, op->ky32, op->kz32,
-                                                                    op->dinv32), v, out, add, status, st);
+                                                                    op->dinv32), v, out, add, status, st, pinned);
     return inner_pcg<float, __nv_bfloat16>(pc, make_stencil<float, __nv_bfloat16>(op, op->d16, op->kx16, op->ky16,
                                                                                    op->kz16, op->dinv16),
-                                           v, out, add, status, st);
+                                           v, out, add, status, st, pinned);
   }
   // Chebyshev
   if (pc->precision == PFK_FP64)
@@ -898,7 +910,6 @@ extern "C" pfk_status pfk_pc_apply_inner_pcg_noalloc(pfk_context* ctx, const pfk
   tmp.kind = PFK_PC_INNER_PCG;
   tmp.inner = inner_iters;
   tmp.precision = PFK_FP64;
-  tmp.separate = true;
   tmp.buf = scratch;
   tmp.buf_bytes = 5 * (size_t)op->n * sizeof(double);
   tmp.partials = scratch + 5 * kNoallocMaxN;
@@ -908,7 +919,8 @@ extern "C" pfk_status pfk_pc_apply_inner_pcg_noalloc(pfk_context* ctx, const pfk
   // must start at zero
   PFK_CUDA(ctx, cudaMemsetAsync(tmp.ctl, 0, sizeof(PcCtl), ctx->stream));
   const StencilT<double, double> A = make_stencil<double, double>(op, op->d, op->kx, op->ky, op->kz, op->dinv);
-  e = inner_pcg<double, double>(&tmp, A, v, y, nullptr, nullptr, ctx->stream);
+  // separate kernels: a cooperative launch may allocate
+  e = inner_pcg<double, double>(&tmp, A, v, y, nullptr, nullptr, ctx->stream, true);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "inner PCG kernels");
   PFK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   return PFK_OK;

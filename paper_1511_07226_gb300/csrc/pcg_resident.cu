@@ -324,7 +324,7 @@ static size_t res_smem_bytes(const pfk_context* ctx, int64_t n) {
 // 96^3 192 -> 147, before the work in the waits), so the memory sets the line.
 bool pcg_resident_fits(const pfk_pc* pc) {
   const int64_t n = pc->op->n;
-  return !pc->separate && n >= 1 && n < INT32_MAX / 2 && res_smem_bytes(pc->ctx, n) <= (size_t)kResSmemLimit &&
+  return n >= 1 && n < INT32_MAX / 2 && res_smem_bytes(pc->ctx, n) <= (size_t)kResSmemLimit &&
          2 * res_blocks(pc->ctx, n) <= pc->partials_cap;
 }
 

@@ -168,8 +168,6 @@ struct pfk_pc {
   pfk::PcCtl* ctl = nullptr;
   double* partials = nullptr;
   int partials_cap = 0;         // doubles in `partials` (bounds the grid of the reduction kernels)
-  bool separate = false;        // inner PCG as separate kernels at every size (the allocation-free entry
-                                // point: a cooperative launch may allocate, and its scratch is shared)
   // noisy preconditioner: the noise bank (count x n) and 1 / ||xi_j||
   double noise_eta = 0.0;
   double* bank = nullptr;
@@ -207,34 +205,37 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // Sums V values of every lane over the warp (V a power of two, at most 32):
-// lane l returns the sum of acc[l % V].  Each step exchanges half of the
-// values a lane still holds with a partner lane, so the warp spends V - 1 (+
-// 5 - log2 V) FP64 additions instead of the 5 V of V shuffle trees: on GB300
-// an FP64 warp instruction holds its pipe for ~76 cycles, and the 160
-// additions of 32 trees cost a resident warp as much as the products of five
-// elements.
+// lane l returns the sum of acc[l / (32 / V)], bitwise warp_sum(acc[j]): the
+// lanes are added in warp_sum's order (16, 8, 4, 2, 1 apart).  Each step
+// exchanges half of the values a lane still holds with a partner lane, so the
+// warp spends V - 1 (+ 5 - log2 V) FP64 additions instead of the 5 V of V
+// shuffle trees: on GB300 an FP64 warp instruction holds its pipe for ~76
+// cycles, and the 160 additions of 32 trees cost a resident warp as much as the
+// products of five elements.
 template <int V>
 __device__ __forceinline__ double warp_sum_transposed(double (&acc)[V]) {
   const int lane = threadIdx.x & 31;
+  int m = 16;
 #pragma unroll
-  for (int h = V / 2; h > 0; h >>= 1) {
-    const bool up = (lane & h) != 0;
+  for (int h = V / 2; h > 0; h >>= 1, m >>= 1) {
+    const bool up = (lane & m) != 0;
 #pragma unroll
     for (int j = 0; j < h; ++j) {
       const double keep = up ? acc[j + h] : acc[j], send = up ? acc[j] : acc[j + h];
-      acc[j] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+      acc[j] = keep + __shfl_xor_sync(0xffffffffu, send, m);
     }
   }
   double v = acc[0];
 #pragma unroll
-  for (int o = V; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (; m > 0; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
   return v;
 }
 
 // Value j of every thread summed over the block (ND values of kThreads
-// threads, staged in buf): warp (blockIdx + j) mod 8 adds the eight warps'
-// values lane by lane and runs one shuffle tree, so a value costs the block 12
-// FP64 instructions instead of 8 trees of 5; the warp rotates with the block
+// threads, staged in buf), bitwise as by a warp_sum in each warp and the warps
+// added in order: warp (blockIdx + j) mod 8 sums the eight warps' values
+// transposed (9 additions) and adds the eight sums (7), so a value costs the
+// block 16 FP64 instructions instead of 48; the warp rotates with the block
 // so that the resident blocks' sums spread over the SM's four FP64 pipes.
 // store(j, sum) is called by lane 0 of that warp.
 template <int ND, typename F>
@@ -246,10 +247,14 @@ __device__ __forceinline__ void block_sums(const double (&acc)[ND], double (&buf
   __syncthreads();
   const int j = (warp - (int)blockIdx.x) & 7;
   if (j < ND) {
-    const double* b = buf[j] + lane;
-    const double v = ((b[0] + b[64]) + (b[128] + b[192])) + ((b[32] + b[96]) + (b[160] + b[224]));
-    const double w = warp_sum(v);
-    if (lane == 0) store(j, w);
+    double b[8];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) b[w] = buf[j][w * 32 + lane];
+    const double s = warp_sum_transposed<8>(b);   // lanes 4 w .. 4 w + 3: the sum of warp w
+    double v = __shfl_sync(0xffffffffu, s, 0);
+#pragma unroll
+    for (int w = 1; w < 8; ++w) v += __shfl_sync(0xffffffffu, s, 4 * w);
+    if (lane == 0) store(j, v);
   }
 }
 
@@ -417,13 +422,11 @@ __device__ __forceinline__ bool reduce_last_block(const double (&acc)[ND], int n
 }
 
 // reduce_last_block for the kernels of the FP64 path (blocks of kThreads
-// threads), with block_sums in place of the shuffle trees: partials[blockIdx.x *
-// ND + j]; the last block's thread t takes rows t, t + kThreads, ..., then
-// block_sums.  At 64^3 the inner PCG's r update went from 9.0 to 5.6 us and
-// s = A p from 10.2 to 8.8 us, most of it the trees of 64 resident warps.  The
-// reductions that also serve the reduced-precision preconditioners and
-// PIPEFGMRES's shift keep reduce_last_block: a last-bit change there moves
-// FP32 roundings downstream.
+// threads), with block_sums in place of the shuffle trees: the same sums bit for
+// bit (partials[blockIdx.x * ND + j]; the last block's thread t takes rows t, t +
+// kThreads, ..., then block_sums).  The order of these sums is part of the
+// methods' results: the pipelined recurrences amplify a last-bit difference by
+// up to 1e8 within some tens of iterations.
 template <int ND>
 __device__ __forceinline__ bool reduce_last_block_fast(const double (&acc)[ND], double* partials, unsigned int* counter,
                                                   double* sums) {
@@ -464,8 +467,10 @@ cudaError_t op_apply(const pfk_operator* op, const double* x, double* y, const d
                      cudaStream_t st);
 
 // out = add + B(v) (add may be null).  `status` as above.
+// pinned: the FP64 inner PCG adds its inner products in one fixed order
+// (pc.cu), for the pipelined recurrences, which amplify a last-bit difference.
 cudaError_t pc_apply(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,
-                     cudaStream_t st);
+                     cudaStream_t st, bool pinned);
 
 // FP64 inner PCG in one cooperative launch (pcg_resident.cu).
 bool pcg_resident_fits(const pfk_pc* pc);

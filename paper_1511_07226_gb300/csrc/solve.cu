@@ -29,12 +29,12 @@
 namespace pfk {
 
 cudaError_t SolveEnv::pc_apply(const double* v, double* out, const double* add, const int* status) const {
-  if (pc) return pfk::pc_apply(pc, v, out, add, status, st);
+  if (pc) return pfk::pc_apply(pc, v, out, add, status, st, pinned);
   pfk_pc id;   // identity
   id.ctx = ctx;
   id.op = op;
   id.kind = PFK_PC_NONE;
-  return pfk::pc_apply(&id, v, out, add, status, st);
+  return pfk::pc_apply(&id, v, out, add, status, st, pinned);
 }
 
 cudaError_t SolveEnv::mark_pass(int which) const {
@@ -217,6 +217,7 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
   env.partials_cap = pd;
   env.N = N;
   env.pass_ev0 = env.pass_ev1 = nullptr;
+  env.pinned = !M->blocking();
 
   long long kernel_launches = 0;
 

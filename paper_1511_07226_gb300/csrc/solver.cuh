@@ -24,6 +24,7 @@ struct SolveEnv {
            (int64_t)(blocks + (blocks + kCombineGroup - 1) / kCombineGroup) * stride <= partials_cap;
   }
   cudaEvent_t pass_ev0, pass_ev1;   // profiling: recorded around the fused pass (or null)
+  bool pinned;               // the preconditioner's sums in the fixed order (pc_apply)
 
   // out = add + B(v); B = identity when pc is null.
   cudaError_t pc_apply(const double* v, double* out, const double* add, const int* status) const;
@@ -49,6 +50,11 @@ class Method {
   virtual cudaError_t end_cycle(const SolveEnv& env, double* x) { (void)env; (void)x; return cudaSuccess; }
   // Iterations one call of iteration() covers at most.
   virtual int iterations_per_step() const { return 1; }
+  // Whether u_i, p_i and s_i are formed from r_i and u_i themselves (FCG, GCR,
+  // FGMRES): a rounding difference of the inner products then stays one.  In the
+  // pipelined recurrences, where no vector is ever formed anew, it grows: by up
+  // to 1e8 in 20 iterations of PIPEGCR at 26^3, contrast 1e3.
+  virtual bool blocking() const { return false; }
   // Number of ring/Hessenberg columns (GMRES types restart after this many).
   virtual int cycle_length() const { return 0; }
   // Once per solve, before bind: picks the persistent single-launch form when

@@ -1,0 +1,81 @@
+"""Solves whose results are pinned bit for bit, and the recording of them.
+
+The pipelined recurrences (PIPEFCG, PIPEGCR, PIPEFGMRES and their variants)
+never form a residual or a preconditioned residual anew, so a last-bit
+difference of one inner product grows within some tens of iterations: 26^3
+PIPEGCR at contrast 1e3 moves by up to 5e-7 in 20.  The order in which their
+kernels add is therefore part of their results.  Inputs are exact (integers and
+powers of two): the same bits wherever they are made.
+
+`python tests/_fixed_order.py OUT.json` (repository root as the working folder, a
+GPU, the library built) records the results that tests/test_gpu_fixed_order.py
+compares with; the recorded ones were made on a GB300 (152 SMs, which the grids
+and so the orders depend on) by the build of commit c2a6e66.
+"""
+import json
+import os
+import sys
+
+import numpy as np
+
+GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "fixed_order.json")
+SAMPLES = 33
+NONE, ADV = (0.0, 0.0, 0.0), (2.0, 1.0, -1.0)
+
+
+def _c(group, method, dims, mmax, maxit, pc="inner_pcg", inner=4, vel=NONE, storage="matrix_free", **kw):
+    return dict(group=group, method=method, dims=dims, mmax=mmax, maxit=maxit, pc=pc, inner=inner, vel=vel,
+                storage=storage, **kw)
+
+
+CASES = {
+    # the FP64 inner PCG: one cell per thread, several, a grid larger than shared memory, 2D, advection, k = 1
+    "pcg_24": _c("pcg", "pipefcg", (24, 20, 18), 30, 24),
+    "pcg_64": _c("pcg", "pipefcg", (64, 60, 44), 30, 16),
+    "pcg_101": _c("pcg", "pipefcg", (101, 97, 93), 8, 12),
+    "pcg_150": _c("pcg", "pipefcg", (150, 92, 85), 16, 10),
+    "pcg_2d": _c("pcg", "pipefcg", (300, 210, 1), 30, 16, inner=5),
+    "pcg_line": _c("pcg", "pipefcg", (2000, 1, 1), 30, 12, inner=1),
+    "pcg_naive": _c("pcg", "pipefcg_naive", (40, 33, 21), 30, 12),
+    "pcg_gcr_w": _c("pcg", "pipegcr_w", (40, 33, 21), 30, 12),
+    "pcg_theta": _c("pcg", "pipefcg_theta", (40, 33, 21), 30, 12),
+    "pcg_adv": _c("pcg", "pipefgmres", (48, 40, 36), 14, 14, inner=3, vel=ADV),
+}
+
+
+def problem(dims, seed):
+    """Viscosities of contrast 2^10 and a right-hand side, exact in binary."""
+    g = np.random.default_rng(seed)
+    n = int(np.prod(dims))
+    eta = np.ldexp(1.0 + g.integers(0, 1 << 20, n) / (1 << 20), g.integers(-5, 5, n).astype(np.int32))
+    return eta, g.integers(-(1 << 20), 1 << 20, n) / float(1 << 30)
+
+
+def solve_case(ctx, name):
+    """[(x, iterations)] of the case."""
+    from paper_1511_07226_gb300 import pfk
+    c = CASES[name]
+    prm = dict(method=c["method"], mmax=c["mmax"], maxit=c["maxit"], rtol=1e-14)
+    dims = c["dims"] if isinstance(c["dims"], list) else [c["dims"]]
+    probs = [problem(d, 7 + j) for j, d in enumerate(dims)]
+    ops = [pfk.Operator.stencil(ctx, d, eta, c["vel"], storage=c["storage"]) for d, (eta, _) in zip(dims, probs)]
+    if c["group"] == "grouped":
+        xs, infos, _ = pfk.solve_grouped(ctx, ops, [b for _, b in probs], pc_kind=c["pc"], inner_iters=c["inner"],
+                                         **prm)
+        return [(x, i["iterations"]) for x, i in zip(xs, infos)]
+    pc = pfk.Preconditioner(ctx, ops[0], c["pc"], inner_iters=c["inner"])
+    x, info, _ = pfk.solve(ctx, ops[0], pc, probs[0][1], **prm)
+    return [(x, info["iterations"])]
+
+
+def summary(results):
+    """Iterations and SAMPLES entries of every solution, exactly."""
+    return [dict(iterations=int(it), x=[float(x[i]).hex() for i in np.linspace(0, x.size - 1, SAMPLES).astype(int)])
+            for x, it in results]
+
+
+if __name__ == "__main__":
+    sys.path.insert(0, os.getcwd())
+    from paper_1511_07226_gb300 import pfk
+    out = {k: summary(solve_case(pfk.Context(0), k)) for k in CASES}
+    json.dump(out, open(sys.argv[1], "w"), indent=0)
