@@ -78,8 +78,8 @@ __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) base_window_dots
   const int ng = mode == kDotsFcg ? 2 : 0;   // <v, r> and <r, r> after the window's dots
   if (threadIdx.x < nu) s_off[threadIdx.x] = (size_t)((i - nu + (int)threadIdx.x) % slots) * (size_t)N;
   __syncthreads();
-  double g0 = 0.0, g1 = 0.0, acc[NW];
-  window_dots<NW>(v, S, s_off, nu, N, acc, [&](int64_t e, double ve) {
+  double g0 = 0.0, g1 = 0.0;
+  const double tot = window_dots<NW>(v, S, s_off, nu, N, [&](int64_t e, double ve) {
     if (ng) {
       const double re = __ldg(&r[e]);
       g0 = fma(ve, re, g0);
@@ -87,7 +87,6 @@ __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) base_window_dots
     }
   });
   {
-    const double tot = warp_sum_transposed<NW>(acc);
     const int nd = nu + ng;
     const int j = lane / (32 / NW);   // the slot whose sum the lane holds
     if (lane % (32 / NW) == 0 && j < nu) s_red[warp * nd + j] = tot;
@@ -593,9 +592,7 @@ __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) fgb_dots(const d
   const int nk = gs->k + 1;           // p_0 .. p_k
   if (threadIdx.x < nk) s_off[threadIdx.x] = (size_t)threadIdx.x * (size_t)N;
   __syncthreads();
-  double acc[NW];
-  window_dots<NW>(z, P, s_off, nk, N, acc, [](int64_t, double) {});
-  const double tot = warp_sum_transposed<NW>(acc);
+  const double tot = window_dots<NW>(z, P, s_off, nk, N, [](int64_t, double) {});
   const int j = lane / (32 / NW);   // the slot whose sum the lane holds
   if (lane % (32 / NW) == 0 && j < nk) s_red[warp * nk + j] = tot;
   __syncthreads();

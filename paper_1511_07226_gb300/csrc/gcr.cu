@@ -23,7 +23,6 @@
 #include "pfk_internal.cuh"
 #include "solver.cuh"
 #include "stencil.cuh"
-#include "stencil_flat.cuh"
 
 namespace pfk {
 
@@ -226,6 +225,16 @@ struct GcrApplyEpi {
   }
 };
 
+// The order of the iteration's sums is fixed: the walk's columns (planes per
+// unit chosen for this many resident blocks per SM: 80 and 96 registers) for
+// gamma, delta and ||r||^2, and a grid of kGcrDotsBlocksPerSm blocks per SM for
+// the window.  The recurrences amplify a last-bit difference of these sums by up
+// to 1e8 within 20 iterations (26^3, contrast 1e3), so forms that add in another
+// order (the operator on flat rows, grids by size) are not used here, although
+// on ragged sides the flat rows are faster (ops.cu).
+constexpr int kWalkBlocksPerSm = 3, kWalkBlocksPerSmAdv = 2;
+constexpr int kGcrDotsBlocksPerSm = 5;
+
 template <bool ADV>
 __global__ void __launch_bounds__(kTileThreads) pipegcr_apply_walk(TiledStencil<double, double> T, GcrArgs a) {
   SolveCtl* ctl = a.ctl;
@@ -241,34 +250,13 @@ __global__ void __launch_bounds__(kTileThreads) pipegcr_apply_walk(TiledStencil<
   }
 }
 
-// The same on the flat rows (64^3, whole tiles: the same time; ragged sides gain as in ops.cu).
-template <bool ADV>
-__global__ void __launch_bounds__(kThreads) pipegcr_apply_flat(FlatStencil A, GcrArgs a) {
-  SolveCtl* ctl = a.ctl;
-  if (ctl->status != kRun) return;
-  GcrApplyEpi e{a.w, a.t, a.r, 0.0, 0.0, 0.0};
-  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
-    const auto pre = e.pre(c);
-    double uc;
-    const double wv = flat_row<ADV>(A, a.u, c, uc);
-    e(c, wv, uc, pre);
-  }
-  double acc[3] = {e.g0, e.g1, e.g2};
-  __shared__ double sums[3];
-  if (reduce_last_block_fast<3>(acc, a.partials, &ctl->counter, sums) && threadIdx.x == 0) {
-    ctl->pend[0] = sums[0];
-    ctl->pend[1] = sums[1];
-    ctl->pend[2] = sums[2];
-  }
-}
-
 // <w_i, s_k> over the window (window_dots); the last block adds the
 // walk's gamma, delta, ||r||^2 and runs the scalar phase of iteration i.
 template <int NW>
-__global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) pipegcr_window_dots(GcrArgs a, int stencil_flops) {
+__global__ void __launch_bounds__(kGcrThreads, kGcrDotsBlocksPerSm) pipegcr_window_dots(GcrArgs a, int stencil_flops) {
   SolveCtl* ctl = a.ctl;
   if (ctl->status != kRun) return;
-  constexpr int NWARPS = kWinThreads / 32;
+  constexpr int NWARPS = kGcrThreads / 32;
   __shared__ size_t s_off[NW];
   __shared__ double s_red[NWARPS * NW];
   __shared__ double s_sum[NW];
@@ -282,9 +270,7 @@ __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) pipegcr_window_d
     s_off[threadIdx.x] = (size_t)(k % slots) * (size_t)N;
   }
   __syncthreads();
-  double acc[NW];
-  window_dots<NW>(a.w, a.S, s_off, nu, N, acc, [](int64_t, double) {});
-  const double tot = warp_sum_transposed<NW>(acc);
+  const double tot = window_dots<NW, true>(a.w, a.S, s_off, nu, N, [](int64_t, double) {});
   const int j = lane / (32 / NW);   // the slot whose sum the lane holds
   if (lane % (32 / NW) == 0 && j < nu) s_red[warp * nu + j] = tot;
   __syncthreads();
@@ -371,30 +357,26 @@ class PipeGcr : public Method {
     if (e != cudaSuccess) return e;
     if (stencil) {
       TiledStencil<double, double> T;
-      const int slots = adv ? tiled_stencil_slots(pipegcr_apply_walk<true>, env.ctx->num_sms)
-                            : tiled_stencil_slots(pipegcr_apply_walk<false>, env.ctx->num_sms);
+      const int slots = (adv ? kWalkBlocksPerSmAdv : kWalkBlocksPerSm) * env.ctx->num_sms;
       const int units = tiled_stencil_setup<double, double>(T, op, op->d, op->kx, op->ky, op->kz, slots);
       const int64_t wcap = env.partials_cap / 3;
       const int wblocks = (int)(units < wcap ? units : wcap);
-      const int sblocks = window_dots_blocks(env.ctx, N_);
+      const int64_t wneed = (N_ + kGcrThreads - 1) / kGcrThreads;
+      const int64_t wslots = (int64_t)env.ctx->num_sms * kGcrDotsBlocksPerSm;
+      const int sblocks = (int)(wneed < wslots ? wneed : wslots);
       if (!env.partials_fit_2l(sblocks, tmpl)) return cudaErrorInvalidValue;
       switch (tmpl) {
         case 8: pipegcr_advance<8><<<ablocks, kThreads, 0, env.st>>>(a); break;
         case 16: pipegcr_advance<16><<<ablocks, kThreads, 0, env.st>>>(a); break;
         default: pipegcr_advance<32><<<ablocks, kThreads, 0, env.st>>>(a); break;
       }
-      if (flat_stencil_fits(op)) {
-        const FlatStencil F = flat_stencil(op);
-        if (!env.partials_fit(ablocks, 3)) return cudaErrorInvalidValue;
-        if (adv) pipegcr_apply_flat<true><<<ablocks, kThreads, 0, env.st>>>(F, a);
-        else pipegcr_apply_flat<false><<<ablocks, kThreads, 0, env.st>>>(F, a);
-      } else if (adv) pipegcr_apply_walk<true><<<wblocks, kTileThreads, 0, env.st>>>(T, a);
+      if (adv) pipegcr_apply_walk<true><<<wblocks, kTileThreads, 0, env.st>>>(T, a);
       else pipegcr_apply_walk<false><<<wblocks, kTileThreads, 0, env.st>>>(T, a);
       const int sf = adv ? 10 : 7;
       switch (tmpl) {
-        case 8: pipegcr_window_dots<8><<<sblocks, kWinThreads, 0, env.st>>>(a, sf); break;
-        case 16: pipegcr_window_dots<16><<<sblocks, kWinThreads, 0, env.st>>>(a, sf); break;
-        default: pipegcr_window_dots<32><<<sblocks, kWinThreads, 0, env.st>>>(a, sf); break;
+        case 8: pipegcr_window_dots<8><<<sblocks, kGcrThreads, 0, env.st>>>(a, sf); break;
+        case 16: pipegcr_window_dots<16><<<sblocks, kGcrThreads, 0, env.st>>>(a, sf); break;
+        default: pipegcr_window_dots<32><<<sblocks, kGcrThreads, 0, env.st>>>(a, sf); break;
       }
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       if ((e = env.mark_pass(1)) != cudaSuccess) return e;

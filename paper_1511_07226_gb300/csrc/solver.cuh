@@ -76,15 +76,16 @@ class Method {
 
 // Window dots, the reduction of the CR types and the base methods: one
 // register accumulator per window slot and thread (independent FMAs, the
-// loads of a whole window in flight), then warp_sum_transposed.  acc[j] +=
-// <v, s_j>; s_off holds the slots' offsets.  body(e, v_e) adds the caller's own
-// products.  The loop is instantiated for window sizes rounded up to 4: with
-// one loop for 32 slots the guarded products of the empty slots were issued all
-// the same (101x97x93: 79 us at every window size).
+// loads of a whole window in flight), then warp_sum_transposed: lane l returns
+// the warp's <v, s_j> for j = l / (32 / NW).  s_off holds the slots' offsets.
+// body(e, v_e) adds the caller's own products.  The loop is instantiated for
+// window sizes rounded up to 4: with one loop for 32 slots the guarded products
+// of the empty slots were issued all the same (101x97x93: 79 us at every window
+// size).  The order of a thread's sum depends on the grid alone.
 constexpr int kWinThreads = 128;
-constexpr int kWinBlocksPerSm = 4;   // 128 registers: no spills at 32 slots
+constexpr int kWinBlocksPerSm = 4;   // base methods: 128 registers
 
-template <int NR, int NW, typename F>
+template <int NR, bool LEAN, int NW, typename F>
 __device__ __forceinline__ void window_dots_loop(const double* __restrict__ v, const double* __restrict__ S,
                                                  const size_t* s_off, int nu, int64_t N, double (&acc)[NW],
                                                  F&& body) {
@@ -93,30 +94,47 @@ __device__ __forceinline__ void window_dots_loop(const double* __restrict__ v, c
 #pragma unroll
     for (int j = 0; j < NR; ++j) {
       // rows below NR - 3 exist; the last ones may not
-      const double sv = (j < NR - 3 || j < nu) ? __ldg(&S[s_off[j] + e]) : 0.0;
-      acc[j] = fma(ve, sv, acc[j]);
+      if constexpr (LEAN) {
+        if (j < nu) acc[j] = fma(ve, __ldg(&S[s_off[j] + e]), acc[j]);
+      } else {
+        const double sv = (j < NR - 3 || j < nu) ? __ldg(&S[s_off[j] + e]) : 0.0;
+        acc[j] = fma(ve, sv, acc[j]);
+      }
     }
     body(e, ve);
   }
 }
 
-template <int NW, typename F>
-__device__ __forceinline__ void window_dots(const double* __restrict__ v, const double* __restrict__ S,
-                                            const size_t* s_off, int nu, int64_t N, double (&acc)[NW], F&& body) {
+// LEAN: every slot guarded, which keeps fewer loads in flight and so fewer
+// registers; for the sizes above 16, in a kernel held to 96 registers (without
+// it 750 bytes of spills).
+template <int NR, bool LEAN, int NW, typename F>
+__device__ __forceinline__ double window_dots_n(const double* __restrict__ v, const double* __restrict__ S,
+                                                const size_t* s_off, int nu, int64_t N, F&& body) {
+  double acc[NW];
 #pragma unroll
   for (int j = 0; j < NW; ++j) acc[j] = 0.0;
-  if (nu <= 4) window_dots_loop<4>(v, S, s_off, nu, N, acc, body);
-  else if (nu <= 8) window_dots_loop<8>(v, S, s_off, nu, N, acc, body);
-  else if constexpr (NW >= 16) {
-    if (nu <= 12) window_dots_loop<12>(v, S, s_off, nu, N, acc, body);
-    else if (nu <= 16) window_dots_loop<16>(v, S, s_off, nu, N, acc, body);
-    else if constexpr (NW >= 32) {
-      if (nu <= 20) window_dots_loop<20>(v, S, s_off, nu, N, acc, body);
-      else if (nu <= 24) window_dots_loop<24>(v, S, s_off, nu, N, acc, body);
-      else if (nu <= 28) window_dots_loop<28>(v, S, s_off, nu, N, acc, body);
-      else window_dots_loop<32>(v, S, s_off, nu, N, acc, body);
+  if constexpr (LEAN) asm("" : "+r"(nu));   // or the branch's lower bound on nu removes the guards
+  window_dots_loop<NR, LEAN>(v, S, s_off, nu, N, acc, body);
+  return warp_sum_transposed<NW>(acc);
+}
+
+template <int NW, bool LEAN = false, typename F>
+__device__ __forceinline__ double window_dots(const double* __restrict__ v, const double* __restrict__ S,
+                                            const size_t* s_off, int nu, int64_t N, F&& body) {
+  if (nu <= 4) return window_dots_n<4, false, NW>(v, S, s_off, nu, N, body);
+  if (nu <= 8 || NW == 8) return window_dots_n<8, false, NW>(v, S, s_off, nu, N, body);
+  if constexpr (NW >= 16) {
+    if (nu <= 12) return window_dots_n<12, false, NW>(v, S, s_off, nu, N, body);
+    if (nu <= 16 || NW == 16) return window_dots_n<16, false, NW>(v, S, s_off, nu, N, body);
+    if constexpr (NW >= 32) {
+      if (nu <= 20) return window_dots_n<20, LEAN, NW>(v, S, s_off, nu, N, body);
+      if (nu <= 24) return window_dots_n<24, LEAN, NW>(v, S, s_off, nu, N, body);
+      if (nu <= 28) return window_dots_n<28, LEAN, NW>(v, S, s_off, nu, N, body);
+      return window_dots_n<32, LEAN, NW>(v, S, s_off, nu, N, body);
     }
   }
+  return 0.0;
 }
 
 // Grid of a window-dots kernel: four elements per thread once that still fills

@@ -40,6 +40,14 @@ CASES = {
     "pcg_gcr_w": _c("pcg", "pipegcr_w", (40, 33, 21), 30, 12),
     "pcg_theta": _c("pcg", "pipefcg_theta", (40, 33, 21), 30, 12),
     "pcg_adv": _c("pcg", "pipefgmres", (48, 40, 36), 14, 14, inner=3, vel=ADV),
+    # PIPEGCR: windows up to 32, the three instantiations, ragged sides, 2D, advection
+    "gcr_64": _c("pipegcr", "pipegcr", (64, 64, 64), 32, 34, pc="jacobi"),
+    "gcr_24": _c("pipegcr", "pipegcr", (24, 20, 18), 30, 24),
+    "gcr_ragged": _c("pipegcr", "pipegcr", (101, 67, 45), 16, 20, pc="jacobi"),
+    "gcr_8": _c("pipegcr", "pipegcr", (33, 35, 37), 8, 12),
+    "gcr_150": _c("pipegcr", "pipegcr", (150, 92, 85), 23, 24, pc="jacobi"),
+    "gcr_2d": _c("pipegcr", "pipegcr", (300, 210, 1), 30, 16),
+    "gcr_adv": _c("pipegcr", "pipegcr", (48, 40, 36), 30, 18, vel=ADV),
 }
 
 
