@@ -354,6 +354,30 @@ __device__ __forceinline__ double grp_d(float v) {
 }
 __device__ __forceinline__ double grp_d(double v) { return v; }
 
+// s = A p on the CTA's cells; returns the thread's part of <s, p>, summed a row
+// per warp: that order is fixed, since another one of this sum changes a
+// pipelined solve's iterates far above rounding (26^3 PIPEGCR, contrast 1e3, 20
+// iterations: 2.4e-9).  FP64: the operator on all lanes first, then the products
+// in a loop of their own, whose idle lanes cost one instruction per cell instead
+// of eight.
+template <typename V>
+__device__ __forceinline__ double grp_apply_dot(const GrpSys& S, const GrpCta* g, const GrpCoef<V>& A, const V* p,
+                                                V* s) {
+  constexpr bool F64 = sizeof(V) == 8;
+  double acc = 0.0;
+  grp_cells<F64>(S, g, [&](int64_t c, int i, int j, int k) {
+    const V sv = grp_row_t<V>(S, A, p, c, i, j, k);
+    s[c] = sv;
+    if (!F64) acc += grp_d(sv) * grp_d(p[c]);
+  });
+  if (F64) {
+    __syncthreads();
+#pragma unroll 2
+    GRP_ROWS(S, g, c, i, j, k) acc += grp_d(s[c]) * grp_d(p[c]);
+  }
+  return acc;
+}
+
 // Inner Jacobi-PCG in V (FP64, or FP32 vectors and coefficient copies with
 // the inner products of FP32 values accumulated in FP64): out = add + x_k.
 template <typename V>
@@ -394,12 +418,7 @@ __device__ void grp_pcg(const GrpSys& S, GrpCta* g, const GrpCoef<V>& A, const d
       GRP_ELEMS(S, g, e) p[e] = dinv[e] * r[e];
       grp_barrier(S, g);
     }
-    double acc[1] = {0.0};
-    grp_cells<F64>(S, g, [&](int64_t c, int i, int j, int k) {
-      const V sv = grp_row_t<V>(S, A, p, c, i, j, k);
-      s[c] = sv;
-      acc[0] += grp_d(sv) * grp_d(p[c]);
-    });
+    double acc[1] = {grp_apply_dot<V>(S, g, A, p, s)};
     grp_sum<1>(S, g, acc, s_red);
     if (threadIdx.x == 0) {
       if (g->red[0] == 0.0) g->last_x = 0;
@@ -452,12 +471,7 @@ __device__ void grp_pcg(const GrpSys& S, GrpCta* g, const GrpCoef<V>& A, const d
     }
     {
       // s_i = A p_i, eta_i
-      double acc[1] = {0.0};
-      grp_cells<F64>(S, g, [&](int64_t c, int i, int j, int k) {
-        const V sv = grp_row_t<V>(S, A, p, c, i, j, k);
-        s[c] = sv;
-        acc[0] += grp_d(sv) * grp_d(p[c]);
-      });
+      double acc[1] = {grp_apply_dot<V>(S, g, A, p, s)};
       grp_sum<1>(S, g, acc, s_red);
       if (threadIdx.x == 0) {
         if (g->red[0] == 0.0) g->last_x = it;

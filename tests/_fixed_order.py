@@ -48,6 +48,10 @@ CASES = {
     "gcr_150": _c("pipegcr", "pipegcr", (150, 92, 85), 23, 24, pc="jacobi"),
     "gcr_2d": _c("pipegcr", "pipegcr", (300, 210, 1), 30, 16),
     "gcr_adv": _c("pipegcr", "pipegcr", (48, 40, 36), 30, 18, vel=ADV),
+    # the grouped kernel
+    "grp_fcg": _c("grouped", "pipefcg", [(26, 26, 26), (40, 37, 33), (31, 17, 5), (64, 9, 1)], 30, 16),
+    "grp_gcr": _c("grouped", "pipegcr", [(26, 26, 26), (40, 37, 33), (31, 17, 5), (64, 9, 1)], 30, 16),
+    "grp_gmres": _c("grouped", "pipefgmres", [(26, 26, 26), (40, 37, 33), (31, 17, 5)], 12, 12, vel=ADV),
 }
 
 
