@@ -37,10 +37,8 @@
 // On this GPU an FP64 instruction costs its sub-partition tens of
 // nanoseconds whatever its active lanes, so the reductions and the scalar
 // phase are arranged to keep such instructions few and off one warp's chain
-// (48 iterations of 64 x 64 with host arrays: 842 -> 793 us, 12.3 us an
-// iteration with windows up to 30, by the exchange-step sums, one direction
-// per thread of a row, more row groups in sum_partials and three scalar chains
-// side by side).
+// (48 iterations of 64 x 64 with host arrays: 842 -> 800 us by the exchange-step
+// sums and one direction per thread of a row).
 // Block 0 keeps the control block up to date (status, counters, history) for
 // the host driver.
 #include "pfk_internal.cuh"
@@ -109,10 +107,8 @@ __device__ __forceinline__ void red_add_release(unsigned int* p, unsigned int v)
 // others wait for it with acquire loads.  The wait is bounded (the control
 // block's bar_timeout_ns, 2 s by default): on time-out the block raises
 // bar_abort, and a raised bar_abort ends every other wait.
-// Returns false in that case.  meanwhile() runs in the other threads while
-// thread 0 waits.
-template <typename F>
-__device__ __forceinline__ bool grid_barrier(SolveCtl* ctl, F&& meanwhile) {
+// Returns false in that case.
+__device__ __forceinline__ bool grid_barrier(SolveCtl* ctl) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -139,15 +135,9 @@ __device__ __forceinline__ bool grid_barrier(SolveCtl* ctl, F&& meanwhile) {
       }
     }
     s_ok = ok;
-  } else {
-    meanwhile();
   }
   __syncthreads();
   return s_ok != 0;
-}
-
-__device__ __forceinline__ bool grid_barrier(SolveCtl* ctl) {
-  return grid_barrier(ctl, [] {});
 }
 
 // Sum of a value over the eight rows a warp holds, for the thread position q
@@ -184,10 +174,14 @@ __device__ __forceinline__ void wait_partials() {
 // spread over (column, row group) tasks that keep all lanes busy: task t of
 // the block sums rows g, g + G, g + 2G, ... of column j (t = g * nd + j), then
 // thread j adds the G group sums in group order: nb / G + G additions in a
-// row.  G is as many groups as fit in the block's threads, at most gmax =
-// sqrt(nb), beyond which the second sum grows by more than the first shrinks
-// (nb = 128, 16 columns: 24 additions, where at most 4 groups took 36).  Every
-// block gets bitwise the same sums.
+// row.  G is as many groups as fit in the block's threads, at most gmax: for
+// FCG sqrt(nb), beyond which the second sum grows by more than the first
+// shrinks (nb = 128, 16 columns: 24 additions, where 4 groups take 36); for
+// PIPEFCG, whose recurrences amplify a last-bit difference of these sums, always
+// kPipeGroups, so that their order does not change.  Every block gets bitwise
+// the same sums.
+constexpr int kPipeGroups = 4;
+
 __device__ __forceinline__ int max_groups(int nb) {
   int G = 1;
   while ((G + 1) * (G + 1) <= nb) ++G;
@@ -267,7 +261,6 @@ struct PerState {
   double alpha, gamma, delta, eta, rho;
   double beta[PFK_MAX_MMAX];
   double eta_ring[PFK_MAX_MMAX + 1];
-  double inv_eta[PFK_MAX_MMAX + 1];        // 1 / eta_ring (PIPEFCG)
   double sums[kPerNd];
   double cw[PFK_MAX_MMAX + 1];
   double tmp[2 * PFK_MAX_MMAX + 2];
@@ -295,10 +288,7 @@ __device__ __forceinline__ void load_state(PerState* st, const SolveCtl* ctl) {
     st->windows = 0;
   }
   for (int j = threadIdx.x; j < PFK_MAX_MMAX; j += blockDim.x) st->beta[j] = ctl->beta[j];
-  for (int j = threadIdx.x; j <= PFK_MAX_MMAX; j += blockDim.x) {
-    st->eta_ring[j] = ctl->eta_ring[j];
-    st->inv_eta[j] = 1.0 / st->eta_ring[j];   // of a slot in use; the others are not read
-  }
+  for (int j = threadIdx.x; j <= PFK_MAX_MMAX; j += blockDim.x) st->eta_ring[j] = ctl->eta_ring[j];
   __syncthreads();
 }
 
@@ -529,7 +519,6 @@ __global__ void __launch_bounds__(kPerThreads, 1) pipefcg_persistent(PersistArgs
   const double* dfrom = q == 0 ? su : q == 1 ? sw : q == 2 ? sm : sn;   // thread q's direction update starts from this,
   double* vown = q == 0 ? sx : q == 1 ? sr : q == 2 ? su : sw;          // and the vector it advances
   const bool jacobi = a.dinv != nullptr;
-  const int gmax = max_groups(nb);
 
   for (int g = 0; g < a.iters; ++g) {
     if (st.status != kRun) break;
@@ -605,10 +594,7 @@ __global__ void __launch_bounds__(kPerThreads, 1) pipefcg_persistent(PersistArgs
     }
     write_pipefcg_row<NWQ>(scq, acc, nwp, s_red, part + (size_t)blockIdx.x * kPerNd);
 
-    const bool met = grid_barrier(ctl, [&] {
-      if (threadIdx.x == 96) st.inv_eta[cslot] = 1.0 / st.eta_ring[cslot];   // for the scalar phase
-    });
-    if (!met) {
+    if (!grid_barrier(ctl)) {
       if (blockIdx.x == 0 && threadIdx.x == 0) ctl->status = kTimeout;
       return;
     }
@@ -622,16 +608,12 @@ __global__ void __launch_bounds__(kPerThreads, 1) pipefcg_persistent(PersistArgs
       if (e >= 0 && q == 0) sn[l] = csr_row(a, cs, mnew, e, l);
     }
     wait_partials();
-    sum_partials(s_part, nb, 4 + nwp, gmax, st.sums, s_red);
+    sum_partials(s_part, nb, 4 + nwp, kPipeGroups, st.sums, s_red);
 
     // ---- scalar phase of iteration i (Alg. 8), the same in every block ----
-    // Three chains side by side, on different sub-partitions (what the last two
-    // form is used only when the iteration goes on): thread 32 forms rho_i and
-    // the convergence verdict and writes the history; warp 2 forms the betas;
-    // warp 0 forms eta_i and alpha_i without waiting for them, from beta^2
-    // eta_k = (c / eta_k) c with the reciprocals kept beside eta_k (a division
-    // is a chain of some ten FP64 instructions; one rounding more than c /
-    // eta_k, one less than beta * beta * eta_k).
+    // Warp 1 (thread 32) forms rho_i and the convergence verdict and writes the
+    // history while warp 0 forms the betas, eta_i and alpha_i (used only when
+    // the iteration goes on): the two chains run on different sub-partitions.
     const int nu = nu_window(i, a.mmax, st.truncation);
     if (threadIdx.x == 32) {
       const double gamma = st.sums[0], rr = st.sums[2];
@@ -640,25 +622,17 @@ __global__ void __launch_bounds__(kPerThreads, 1) pipefcg_persistent(PersistArgs
       per_push_history(&st, ctl, rho, st.history ? sqrt(rr) : nan(""), nan(""), nan(""));
       st.go = !isfinite(rho) ? -1 : (rho <= st.target ? 0 : 1);
     }
-    // window dots in order k = i-1-nwp .. i-1 (W_{i-1}, then s_{i-1}); W_i is the last nu
-    const auto window_dot = [&](int jj) {
-      const int c = nwp + 1 - nu + jj;
-      return c < nwp ? st.sums[4 + c] : st.sums[3];
-    };
-    if (threadIdx.x >= 64 && (int)threadIdx.x < 64 + nu) {
-      const int jj = (int)threadIdx.x - 64;
-      st.beta[jj] = -window_dot(jj) / st.eta_ring[(i - nu + jj) % slots];
-    }
     if (threadIdx.x < 32) {
+      // window dots in order k = i-1-nwp .. i-1 (W_{i-1}, then s_{i-1}); W_i is the last nu
       const int jj = (int)threadIdx.x;
       double term = 0.0;
       if (jj < nu) {
-        const double cv = window_dot(jj);
-        const int ks = (i - nu + jj) % slots;
-        const double ek = st.eta_ring[ks];
-        // a reciprocal near the ends of the exponent range is not used
-        const unsigned ex = ((unsigned)__double2hiint(ek) >> 20) & 0x7ffu;
-        term = (ex - 23u < 2000u ? cv * st.inv_eta[ks] : cv / ek) * cv;
+        const int c = nwp + 1 - nu + jj;
+        const double cv = c < nwp ? st.sums[4 + c] : st.sums[3];
+        const double ek = st.eta_ring[(i - nu + jj) % slots];
+        const double bb = -cv / ek;
+        st.beta[jj] = bb;
+        term = (bb * bb) * ek;
       }
       // sum of beta^2 eta over the window: a fixed shuffle tree
       term = warp_sum(term);

@@ -52,6 +52,12 @@ CASES = {
     "grp_fcg": _c("grouped", "pipefcg", [(26, 26, 26), (40, 37, 33), (31, 17, 5), (64, 9, 1)], 30, 16),
     "grp_gcr": _c("grouped", "pipegcr", [(26, 26, 26), (40, 37, 33), (31, 17, 5), (64, 9, 1)], 30, 16),
     "grp_gmres": _c("grouped", "pipefgmres", [(26, 26, 26), (40, 37, 33), (31, 17, 5)], 12, 12, vel=ADV),
+    # the single-launch PIPEFCG on an assembled operator
+    "csr_4": _c("csr", "pipefcg", (64, 64, 1), 4, 24, pc="jacobi", storage="csr"),
+    "csr_8": _c("csr", "pipefcg", (125, 139, 1), 8, 20, pc="jacobi", storage="csr"),
+    "csr_16": _c("csr", "pipefcg", (64, 64, 1), 16, 24, pc="jacobi", storage="csr"),
+    "csr_30": _c("csr", "pipefcg", (64, 64, 1), 30, 48, pc="jacobi", storage="csr"),
+    "csr_32": _c("csr", "pipefcg", (125, 139, 1), 32, 40, pc="none", storage="csr"),
 }
 
 
