@@ -288,6 +288,7 @@ class PipeFcg : public Method {
   }
 
   double* scratch() override { return tmp_; }
+  int iterations_per_step() const override { return persistent_ ? kPersistentIters : 1; }
 
   bool configure(const pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc, int64_t N, int mode) override {
     persistent_ = mode != 1 && persistent_eligible(ctx, op, pc, PFK_PIPEFCG, naive_ || gcrw_ || theta_, N);
