@@ -228,7 +228,10 @@ typedef struct {
 pfk_status pfk_create_block_preconditioner(pfk_context* ctx, const pfk_operator* K, const pfk_operator* Bt,
                                            const double* schur_diag, const pfk_inner_solve* inner, pfk_pc** pc);
 pfk_status pfk_destroy_preconditioner(pfk_pc* pc);
-/* y = B(v); device pointers of length n, must not overlap. */
+/* y = B(v); device pointers of length n, must not overlap.  PFK_ERR_TIMEOUT (y
+ * not usable) when a grid-barrier wait of the FP64 inner PCG, one launch up to
+ * about 1.03 M unknowns, has not ended after 2 s; the next application starts
+ * afresh. */
 pfk_status pfk_pc_apply(pfk_context* ctx, const pfk_pc* pc, const double* v, double* y);
 
 /* ------------------------------------------------------------------------ */
@@ -271,7 +274,9 @@ pfk_status pfk_pc_apply(pfk_context* ctx, const pfk_pc* pc, const double* v, dou
  *              eligible).  A barrier wait that gives up (barrier_timeout_us)
  *              ends the solve with PFK_ERR_TIMEOUT.
  *  barrier_timeout_us  bound of each grid-barrier wait of the persistent
- *              path: 0 = 2 s; > 0 = that many microseconds; < 0 = no wait
+ *              path, and of the FP64 inner PCG where FCG, GCR and FGMRES run it
+ *              as one launch (up to about 1.03 M unknowns): 0 = 2 s; > 0 = that
+ *              many microseconds; < 0 = no wait
  *              allowed (a barrier that has to wait fails at once: the solve
  *              ends with PFK_ERR_TIMEOUT and the context stays usable -- for
  *              testing the time-out path). */

@@ -85,10 +85,11 @@ pfk_status pfk_create_context(int device, void* cuda_stream, pfk_context** out) 
     pfk_destroy_context(ctx);
     return cuda_fail(nullptr, e, "cudaStreamCreate (capture stream)");
   }
-  if ((e = cudaMallocHost((void**)&ctx->pinned, 2 * sizeof(SolveCtl) + 2 * sizeof(double))) != cudaSuccess) {
+  if ((e = cudaMallocHost((void**)&ctx->pinned, sizeof(HostWords))) != cudaSuccess) {
     pfk_destroy_context(ctx);
     return cuda_fail(nullptr, e, "cudaMallocHost (status words)");
   }
+  ctx->pinned->pc_gave_up = 0u;
   // stream-ordered: no device-wide synchronisation, so a context can be created
   // while another thread records a CUDA graph
   if ((e = cudaMemsetAsync(ctx->scratch_counter, 0, 4 * sizeof(unsigned int), ctx->stream)) != cudaSuccess ||
@@ -270,9 +271,10 @@ pfk_status pfk_pc_apply(pfk_context* ctx, const pfk_pc* pc, const double* v, dou
   CHECK_ARG(ctx, ctx && pc && v && y, "NULL argument");
   CHECK_ARG(ctx, v != y, "v and y must not overlap");
   cudaSetDevice(ctx->device);
-  PFK_CUDA(ctx, pc_apply(pc, v, y, nullptr, nullptr, ctx->stream, false));
+  PFK_CUDA(ctx, pc_apply(pc, v, y, nullptr, nullptr, ctx->stream,
+                         PcCall{false, kBarrierTimeoutNs, &ctx->pinned->pc_gave_up}));
   PFK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  return PFK_OK;
+  return pc_barrier_recover(ctx, pc, ctx->stream) ? PFK_ERR_TIMEOUT : PFK_OK;
 }
 
 pfk_status pfk_pc_workspace_bytes(const pfk_pc* pc, int64_t* bytes) {

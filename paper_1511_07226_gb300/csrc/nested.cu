@@ -93,7 +93,7 @@ cudaError_t nested_apply(const pfk_pc* pc, const double* v, double* out, const d
   env.partials_cap = S->partials_cap;
   env.N = S->nu;
   env.pass_ev0 = env.pass_ev1 = nullptr;
-  env.pinned = true;
+  env.pcc = PcCall{true, 0, nullptr};   // (the inner preconditioner is Jacobi: no sums, no waits)
   if ((e = S->M->fill(env, S->t, S->y)) != cudaSuccess) return e;                    // K y_u = t_u from 0
   for (int i = 0; i < S->maxit; ++i)
     if ((e = S->M->iteration(env, S->y)) != cudaSuccess) return e;

@@ -549,10 +549,11 @@ constexpr int kPcgWalkBlocksPerSm = 3;
 // rows and half the reducing blocks (150 x 141 x 133: 402 -> 378 us).
 template <typename V, typename C>
 static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v, double* out, const double* add,
-                             const int* status, cudaStream_t st, bool pinned) {
+                             const int* status, cudaStream_t st, const PcCall& how) {
   constexpr bool F64 = std::is_same<V, double>::value;
+  const bool pinned = how.pinned;
   if constexpr (F64) {
-    if (!pinned && pcg_resident_fits(pc)) return pcg_resident(pc, v, out, add, status, st);
+    if (!pinned && pcg_resident_fits(pc)) return pcg_resident(pc, v, out, add, status, st, how);
   }
   const int64_t n = A.n;
   V* base = (V*)pc->buf;
@@ -691,7 +692,7 @@ static cudaError_t chebyshev(const pfk_pc* pc, StencilT<V, C> A, const double* v
 }
 
 cudaError_t pc_apply(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,
-                     cudaStream_t st, bool pinned) {
+                     cudaStream_t st, const PcCall& how) {
   if (pc->kind == PFK_PC_BLOCK_UPPER) return nested_apply(pc, v, out, add, status, st);
   const pfk_operator* op = pc->op;
   const int64_t n = op->n;
@@ -711,13 +712,13 @@ cudaError_t pc_apply(const pfk_pc* pc, const double* v, double* out, const doubl
   if (pc->kind == PFK_PC_INNER_PCG) {
     if (pc->precision == PFK_FP64)
       return inner_pcg<double, double>(pc, make_stencil<double, double>(op, op->d, op->kx, op->ky, op->kz, op->dinv),
-                                       v, out, add, status, st, pinned);
+                                       v, out, add, status, st, how);
     if (pc->precision == PFK_FP32)
       return inner_pcg<float, float>(pc, make_stencil<float, float>(op, op->d32, op->kx32, op->ky32, op->kz32,
-                                                                    op->dinv32), v, out, add, status, st, pinned);
+                                                                    op->dinv32), v, out, add, status, st, how);
     return inner_pcg<float, __nv_bfloat16>(pc, make_stencil<float, __nv_bfloat16>(op, op->d16, op->kx16, op->ky16,
                                                                                    op->kz16, op->dinv16),
-                                           v, out, add, status, st, pinned);
+                                           v, out, add, status, st, how);
   }
   // Chebyshev
   if (pc->precision == PFK_FP64)
@@ -920,7 +921,7 @@ extern "C" pfk_status pfk_pc_apply_inner_pcg_noalloc(pfk_context* ctx, const pfk
   PFK_CUDA(ctx, cudaMemsetAsync(tmp.ctl, 0, sizeof(PcCtl), ctx->stream));
   const StencilT<double, double> A = make_stencil<double, double>(op, op->d, op->kx, op->ky, op->kz, op->dinv);
   // separate kernels: a cooperative launch may allocate
-  e = inner_pcg<double, double>(&tmp, A, v, y, nullptr, nullptr, ctx->stream, true);
+  e = inner_pcg<double, double>(&tmp, A, v, y, nullptr, nullptr, ctx->stream, PcCall{true, 0, nullptr});
   if (e != cudaSuccess) return cuda_fail(ctx, e, "inner PCG kernels");
   PFK_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   return PFK_OK;

@@ -25,9 +25,13 @@
 // block 64^3 takes 83 us, but a burst of small solves on several workers 29 ms
 // instead of 21.
 //
-// Every wait is bounded (2 s): a wait that runs out raises an abort word that
-// ends all other waits, and the output is set to NaN.
+// Every wait is bounded (pfk_solve_params' barrier_timeout_us, else 2 s): a wait
+// that runs out raises an abort word that ends all other waits, the blocks that
+// saw it write NaN, and a host-pinned word tells the host, which reports
+// PFK_ERR_TIMEOUT and resets the barrier words before the next application.
 #include "pfk_internal.cuh"
+
+#include <cstddef>
 
 namespace pfk {
 
@@ -35,7 +39,6 @@ constexpr int kResThreads = 512;
 constexpr int kResSmemLimit = 220 * 1024;         // dynamic shared memory of a block (of 227 KB in all)
 constexpr int kResCellBytes = 4 * 8 + 1;          // r, s, x, p and the neighbour flags
 constexpr int kResMinCells = 256;                 // cells per block before the grid is grown
-constexpr long long kResTimeoutNs = 2000000000ll;
 
 struct ResArgs {
   const double* d;
@@ -55,6 +58,8 @@ struct ResArgs {
   PcCtl* ctl;
   int k;
   const int* status;
+  long long bar_timeout_ns;
+  unsigned int* gave_up;   // host-pinned
 };
 
 namespace {
@@ -77,7 +82,8 @@ __device__ __forceinline__ unsigned long long res_ns() {
 // this barrier, counted by the caller, so arriving needs no load, and a wait
 // polls one word: reading the timer and the abort word on every poll as well
 // tripled the time to notice a release.  False when a wait gave up.
-__device__ __forceinline__ bool res_arrive_wait(PcCtl* ctl, unsigned gen) {
+__device__ __forceinline__ bool res_arrive_wait(const ResArgs& a, unsigned gen) {
+  PcCtl* ctl = a.ctl;
   unsigned old;
   asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(&ctl->bar_count) : "memory");
   if (old == gridDim.x - 1) {
@@ -87,11 +93,11 @@ __device__ __forceinline__ bool res_arrive_wait(PcCtl* ctl, unsigned gen) {
   }
   unsigned long long t0 = 0ull;
   for (unsigned polls = 1; res_ld_acquire(&ctl->bar_gen) == gen; ++polls) {
-    if (polls & 63u) continue;
+    if ((polls & 63u) && a.bar_timeout_ns > 0) continue;
     if (res_ld_acquire(&ctl->bar_abort)) return false;
     const unsigned long long t = res_ns();
     if (t0 == 0ull) t0 = t;
-    if (t - t0 > (unsigned long long)kResTimeoutNs) {
+    if (a.bar_timeout_ns <= 0 || t - t0 > (unsigned long long)a.bar_timeout_ns) {
       atomicExch(&ctl->bar_abort, 1u);
       return false;
     }
@@ -113,7 +119,7 @@ template <typename G>
 __device__ __forceinline__ bool res_barrier(const ResArgs& a, ResShared& sh, G&& meanwhile) {
   __syncthreads();
   if (threadIdx.x >= 32) meanwhile((int)threadIdx.x - 32, kResThreads - 32);
-  else if (threadIdx.x == 0) sh.ok = res_arrive_wait(a.ctl, sh.gen++);
+  else if (threadIdx.x == 0) sh.ok = res_arrive_wait(a, sh.gen++);
   __syncthreads();
   return sh.ok != 0;
 }
@@ -144,7 +150,7 @@ __device__ __forceinline__ bool res_sum(const ResArgs& a, ResShared& sh, double 
     int ok = 1;
     if (lane == 0) {
       part[blockIdx.x] = (sh.part[0] + sh.part[1]) + (sh.part[2] + sh.part[3]);
-      ok = res_arrive_wait(a.ctl, sh.gen++);
+      ok = res_arrive_wait(a, sh.gen++);
     }
     ok = __shfl_sync(0xffffffffu, ok, 0);
     double t[8];
@@ -297,6 +303,10 @@ __global__ void __launch_bounds__(kResThreads, 2) pcg_resident_kernel(ResArgs a)
       if (!(ok = res_barrier(a, sh, inner_terms))) break;
     }
   }
+  if (!ok && threadIdx.x == 0) {
+    *(volatile unsigned int*)a.gave_up = 1u;
+    __threadfence_system();
+  }
   // out = add + x_k
 #pragma unroll 4
   for (int q = threadIdx.x; q < cells; q += kResThreads) {
@@ -329,7 +339,7 @@ bool pcg_resident_fits(const pfk_pc* pc) {
 }
 
 cudaError_t pcg_resident(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,
-                         cudaStream_t st) {
+                         cudaStream_t st, const PcCall& how) {
   const pfk_operator* op = pc->op;
   ResArgs a;
   a.d = op->d; a.kx = op->kx; a.ky = op->ky; a.kz = op->kz; a.dinv = op->dinv;
@@ -343,6 +353,8 @@ cudaError_t pcg_resident(const pfk_pc* pc, const double* v, double* out, const d
   a.ctl = pc->ctl;
   a.k = pc->inner;
   a.status = status;
+  a.bar_timeout_ns = how.bar_timeout_ns;
+  a.gave_up = how.gave_up;
   const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
   const void* fn = adv ? (const void*)pcg_resident_kernel<true> : (const void*)pcg_resident_kernel<false>;
   const int smem = (int)res_smem_bytes(pc->ctx, a.n);
@@ -360,6 +372,16 @@ cudaError_t pcg_resident(const pfk_pc* pc, const double* v, double* out, const d
   cfg.numAttrs = 1;
   void* params[] = {&a};
   return cudaLaunchKernelExC(&cfg, fn, params);
+}
+
+bool pc_barrier_recover(pfk_context* ctx, const pfk_pc* pc, cudaStream_t st) {
+  volatile unsigned int* w = &ctx->pinned->pc_gave_up;
+  if (!*w) return false;
+  *w = 0u;
+  static_assert(offsetof(PcCtl, bar_pad) == offsetof(PcCtl, bar_count) + 3 * sizeof(unsigned int), "one range");
+  if (pc->ctl) cudaMemsetAsync(&pc->ctl->bar_count, 0, 4 * sizeof(unsigned int), st);
+  set_error(ctx, "a grid-barrier wait of the inner PCG timed out");
+  return true;
 }
 
 }  // namespace pfk

@@ -89,8 +89,24 @@ struct PcCtl {
   long long row;           // noisy preconditioner: j mod count of the current application
   unsigned int bar_count;  // grid barrier of the resident inner PCG: arrivals,
   unsigned int bar_gen;    // generation,
-  unsigned int bar_abort;  // set when a wait timed out
+  unsigned int bar_abort;  // set when a wait timed out (until pc_barrier_recover)
   unsigned int bar_pad;
+};
+
+// What the host reads without a copy of its own (host-pinned).
+struct HostWords {
+  SolveCtl status[2];        // status copies of pfk_solve
+  double scalars[2];         // <b, b>, <b - A x, b - A x>
+  unsigned int pc_gave_up;   // set by a resident inner PCG whose barrier wait ran out
+};
+
+constexpr long long kBarrierTimeoutNs = 2000000000ll;   // barrier waits by default
+
+// How a preconditioner application adds and waits (FP64 inner PCG).
+struct PcCall {
+  bool pinned;               // inner products in one fixed order (pc.cu), for the pipelined recurrences
+  long long bar_timeout_ns;  // bound of each grid-barrier wait (<= 0: no wait allowed)
+  unsigned int* gave_up;     // host-pinned: set when a wait ran out
 };
 
 }  // namespace pfk
@@ -111,7 +127,7 @@ struct pfk_context {
   double* scratch_partials = nullptr;   // reduction partials for standalone calls
   unsigned int* scratch_counter = nullptr;
   double* scratch_out = nullptr;
-  pfk::SolveCtl* pinned = nullptr;      // host-pinned: two status copies of pfk_solve and two scalars
+  pfk::HostWords* pinned = nullptr;
   // block sizes autotuned by pfk_solve_batched, keyed by (mmax template, log2 of
   // the largest system, count bucket, preconditioner precision + 2 x inner iterations)
   std::map<std::tuple<int, int, int, int>, int> batched_tuned;
@@ -467,15 +483,18 @@ cudaError_t op_apply(const pfk_operator* op, const double* x, double* y, const d
                      cudaStream_t st);
 
 // out = add + B(v) (add may be null).  `status` as above.
-// pinned: the FP64 inner PCG adds its inner products in one fixed order
-// (pc.cu), for the pipelined recurrences, which amplify a last-bit difference.
 cudaError_t pc_apply(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,
-                     cudaStream_t st, bool pinned);
+                     cudaStream_t st, const PcCall& how);
 
 // FP64 inner PCG in one cooperative launch (pcg_resident.cu).
 bool pcg_resident_fits(const pfk_pc* pc);
 cudaError_t pcg_resident(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,
-                         cudaStream_t st);
+                         cudaStream_t st, const PcCall& how);
+
+// After a synchronisation with an application's stream: whether one of its
+// barrier waits ran out.  If so, the barrier is made usable again (in stream
+// order) and the error message set.
+bool pc_barrier_recover(pfk_context* ctx, const pfk_pc* pc, cudaStream_t st);
 
 // Nested block preconditioner (nested.cu).
 cudaError_t nested_apply(const pfk_pc* pc, const double* v, double* out, const double* add, const int* status,

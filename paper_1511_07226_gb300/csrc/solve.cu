@@ -29,12 +29,12 @@
 namespace pfk {
 
 cudaError_t SolveEnv::pc_apply(const double* v, double* out, const double* add, const int* status) const {
-  if (pc) return pfk::pc_apply(pc, v, out, add, status, st, pinned);
+  if (pc) return pfk::pc_apply(pc, v, out, add, status, st, pcc);
   pfk_pc id;   // identity
   id.ctx = ctx;
   id.op = op;
   id.kind = PFK_PC_NONE;
-  return pfk::pc_apply(&id, v, out, add, status, st, pinned);
+  return pfk::pc_apply(&id, v, out, add, status, st, pcc);
 }
 
 cudaError_t SolveEnv::mark_pass(int which) const {
@@ -203,7 +203,7 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
   h.atol = prm->atol;
   h.history = hist;
   h.hist_cap = hist_cap;
-  h.bar_timeout_ns = prm->barrier_timeout_us == 0 ? 2000000000ll
+  h.bar_timeout_ns = prm->barrier_timeout_us == 0 ? kBarrierTimeoutNs
                      : prm->barrier_timeout_us < 0 ? 0ll : 1000ll * (long long)prm->barrier_timeout_us;
   PFK_CUDA(ctx, cudaMemcpyAsync(ctl, &h, sizeof(SolveCtl), cudaMemcpyHostToDevice, st));
 
@@ -217,12 +217,12 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
   env.partials_cap = pd;
   env.N = N;
   env.pass_ev0 = env.pass_ev1 = nullptr;
-  env.pinned = !M->blocking();
+  env.pcc = PcCall{!M->blocking(), h.bar_timeout_ns, &ctx->pinned->pc_gave_up};
 
   long long kernel_launches = 0;
 
-  SolveCtl* hc = ctx->pinned;   // pinned status copies (owned by the context)
-  double* h_bb = reinterpret_cast<double*>(hc + 2);   // pinned: <b, b>, <b - A x, b - A x>
+  SolveCtl* hc = ctx->pinned->status;
+  double* h_bb = ctx->pinned->scalars;
 
   // ---- ||b||: read after the first synchronisation below ----
   PFK_CUDA(ctx, dot_into(ctx, b, b, N, d_out, st));
@@ -385,9 +385,11 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
     }
     if (status == kRun) status = cur.status;
     if (status == kRun && cur.it >= prm->maxit) status = kMaxit;   // a fill stopped short of its first iteration
+    // (the NaN of a preconditioner application whose wait ran out reads as kNonFinite)
+    if (pc && *(volatile unsigned int*)env.pcc.gave_up) status = kTimeout;
     // GMRES types: least-squares solve over the cycle's valid columns and
     // x = x_0 + U y, whatever ended the cycle
-    if (gmres && status != kNonFinite) {
+    if (gmres && status != kNonFinite && status != kTimeout) {
       PFK_CUDA(ctx, M->end_cycle(env, x));
       kernel_launches += 2;
     }
@@ -438,7 +440,7 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
       result = PFK_ERR_BREAKDOWN;
       break;
     }
-    if (status == kTimeout) {
+    if (status == kTimeout) {   // (the inner PCG's: pc_barrier_recover replaces the message)
       set_error(ctx, "a grid-barrier wait of the persistent kernel timed out");
       result = PFK_ERR_TIMEOUT;
       break;
@@ -460,6 +462,7 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
     rnorm_true = rt;
   }
   PFK_CUDA(ctx, cudaStreamSynchronize(st));
+  if (pc && pc_barrier_recover(ctx, pc, st)) result = PFK_ERR_TIMEOUT;
   float ms = 0.f;
   PFK_CUDA(ctx, cudaEventElapsedTime(&ms, tev.v[0], tev.v[1]));
   const int hl = cur.hist_len;

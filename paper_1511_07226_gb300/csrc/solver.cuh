@@ -24,7 +24,7 @@ struct SolveEnv {
            (int64_t)(blocks + (blocks + kCombineGroup - 1) / kCombineGroup) * stride <= partials_cap;
   }
   cudaEvent_t pass_ev0, pass_ev1;   // profiling: recorded around the fused pass (or null)
-  bool pinned;               // the preconditioner's sums in the fixed order (pc_apply)
+  PcCall pcc;                // how the preconditioner adds and waits
 
   // out = add + B(v); B = identity when pc is null.
   cudaError_t pc_apply(const double* v, double* out, const double* add, const int* status) const;
