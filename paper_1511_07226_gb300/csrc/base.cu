@@ -14,7 +14,13 @@
 
 namespace pfk {
 
-static_assert(kWinBlocksPerSm <= kMaxBlocksPerSm, "partials are sized for kMaxBlocksPerSm blocks per SM");
+// Window dots with a pinned order (SolveEnv::pcc): a warp's 32 elements one after
+// the other, lane j holding slot j, the vectors transposed through shared memory.
+constexpr int kPinThreads = 128;
+constexpr int kPinBlocksPerSm = 6;
+constexpr int kPinStride = kPinThreads + 1;
+static_assert(kWinBlocksPerSm <= kMaxBlocksPerSm && kPinBlocksPerSm <= kMaxBlocksPerSm,
+              "partials are sized for kMaxBlocksPerSm blocks per SM");
 
 // A CSR operator (stencil operators take the tiled walk).
 struct CsrView {
@@ -53,11 +59,66 @@ __global__ void __launch_bounds__(kThreads) base_advance(double* __restrict__ x,
   }
 }
 
+template <int NW, typename F>
+__device__ __forceinline__ double window_dots_pinned(const double* __restrict__ v, const double* __restrict__ S,
+                                                     const size_t* s_off, int nu, int64_t N, F&& body) {
+  __shared__ double s_sk[NW * kPinStride];
+  __shared__ double s_v[kPinThreads];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double* my = s_sk + threadIdx.x;
+  const double* wv = s_v + warp * 32;
+  const double* lrow = s_sk + lane * kPinStride + warp * 32;
+  double gw = 0.0;
+  for (int64_t base = (int64_t)blockIdx.x * kPinThreads; base < N; base += (int64_t)gridDim.x * kPinThreads) {
+    const int64_t e = base + threadIdx.x;
+    double vv = 0.0;
+    if (e < N) {
+      vv = v[e];
+      body(e, vv);
+    }
+#pragma unroll
+    for (int j = 0; j < NW; ++j)
+      if (j < nu) my[j * kPinStride] = e < N ? S[s_off[j] + e] : 0.0;
+    s_v[threadIdx.x] = vv;
+    __syncwarp();
+    if (lane < nu) {
+      double c = gw;
+#pragma unroll 8
+      for (int t = 0; t < 32; ++t) c = fma(wv[t], lrow[t], c);
+      gw = c;
+    }
+    __syncwarp();
+  }
+  return gw;
+}
+
 // Dots of a vector v with r (<v, r>), of r with itself, and with the stored
-// s_k of the window W_i (window_dots).  Mode FCG: v = u = B(r_i): convergence
-// test on gamma_i = <u_i, r_i>, then the betas.  Mode GCR: v = A u_i: the betas
-// only.
+// s_k of the window W_i.  Mode FCG: v = u = B(r_i): convergence test on gamma_i =
+// <u_i, r_i>, then the betas.  Mode GCR: v = A u_i: the betas only.
 enum { kDotsFcg = 0, kDotsGcr = 1 };
+
+// The scalar step after the dots (all threads of the last block): c the
+// window's, gamma and rr (FCG) <v, r> and <r, r>.
+__device__ __forceinline__ void base_window_scalars(SolveCtl* ctl, int i, int nu, int slots, int mode,
+                                                    const double* c, double gamma, double rr) {
+  // beta_{i,k} = -<v, s_k> / eta_k, one division per thread (a serial loop of
+  // nu divisions in one thread took 25-30 us at nu = 30); not used when the
+  // iteration stops here
+  if ((int)threadIdx.x < nu)
+    ctl->beta[threadIdx.x] = -c[threadIdx.x] / ctl->eta_ring[(i - nu + (int)threadIdx.x) % slots];
+  if (threadIdx.x != 0) return;
+  ctl->nw = nu;
+  if (mode == kDotsFcg) {
+    // Alg. 2: gamma_i = <u_i, r_i>, convergence
+    ctl->it += 1;
+    ctl->gamma = gamma;
+    const double rho = cgcr_rho(ctl, gamma, rr);
+    ctl->rho = rho;
+    push_history(ctl, rho, sqrt(rr), nan(""), nan(""));
+    if (!isfinite(rho)) { ctl->status = kNonFinite; return; }
+    if (rho <= ctl->target) { ctl->status = kConverged; ctl->i = i; return; }
+  }
+}
 
 template <int NW>
 __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) base_window_dots(const double* __restrict__ v,
@@ -98,24 +159,42 @@ __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) base_window_dots
     __syncthreads();
   }
   if (!combine_block_partials_2l(s_red, nu + ng, partials, ND, &ctl->counter, ctl->gcounter, s_sum)) return;
-  // beta_{i,k} = -<v, s_k> / eta_k, one division per thread (a serial loop of
-  // nu divisions in one thread took 25-30 us at nu = 30); not used when the
-  // iteration stops here
-  if ((int)threadIdx.x < nu)
-    ctl->beta[threadIdx.x] = -s_sum[threadIdx.x] / ctl->eta_ring[(i - nu + (int)threadIdx.x) % slots];
-  if (threadIdx.x != 0) return;
-  ctl->nw = nu;
-  if (mode == kDotsFcg) {
-    // Alg. 2: gamma_i = <u_i, r_i>, convergence
-    const double gamma = s_sum[nu], rr = s_sum[nu + 1];
-    ctl->it += 1;
-    ctl->gamma = gamma;
-    const double rho = cgcr_rho(ctl, gamma, rr);
-    ctl->rho = rho;
-    push_history(ctl, rho, sqrt(rr), nan(""), nan(""));
-    if (!isfinite(rho)) { ctl->status = kNonFinite; return; }
-    if (rho <= ctl->target) { ctl->status = kConverged; ctl->i = i; return; }
+  base_window_scalars(ctl, i, nu, slots, mode, s_sum, s_sum[nu], s_sum[nu + 1]);
+}
+
+// The same with the pinned order.
+template <int NW>
+__global__ void __launch_bounds__(kPinThreads, kPinBlocksPerSm) base_window_dots_pinned(
+    const double* __restrict__ v, const double* __restrict__ r, const double* __restrict__ S, int64_t N,
+    SolveCtl* ctl, double* partials, int mode) {
+  if (ctl->status != kRun) return;
+  constexpr int ND = NW + 2;
+  constexpr int NWARPS = kPinThreads / 32;
+  __shared__ size_t s_off[NW];
+  __shared__ double s_red[NWARPS * ND];
+  __shared__ double s_sum[ND];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = ctl->i + 1;
+  const int nu = nu_window(i, ctl->mmax, ctl->truncation);
+  const int slots = ctl->mmax + 1;
+  if (threadIdx.x < nu) s_off[threadIdx.x] = (size_t)((i - nu + (int)threadIdx.x) % slots) * (size_t)N;
+  __syncthreads();
+  double g0 = 0.0, g1 = 0.0;
+  const double gw = window_dots_pinned<NW>(v, S, s_off, nu, N, [&](int64_t e, double ve) {
+    const double re = r[e];
+    g0 = fma(ve, re, g0);
+    g1 = fma(re, re, g1);
+  });
+  const double w0 = warp_sum(g0), w1 = warp_sum(g1);
+  const int nd = nu + 2;
+  if (lane == 0) {
+    s_red[warp * nd + 0] = w0;
+    s_red[warp * nd + 1] = w1;
   }
+  if (lane < nu) s_red[warp * nd + 2 + lane] = gw;
+  __syncthreads();
+  if (!combine_block_partials_2l(s_red, nd, partials, ND, &ctl->counter, ctl->gcounter, s_sum)) return;
+  base_window_scalars(ctl, i, nu, slots, mode, s_sum + 2, s_sum[0], s_sum[1]);
 }
 
 // p_i = u + sum_k beta_{i,k} p_k over W_i, into ring slot i.
@@ -227,13 +306,13 @@ __global__ void __launch_bounds__(kThreads) base_apply_dots(CsrView A, double* _
     D::add(acc, p[e], sv, D::nd == 3 ? r[e] : 0.0);
   }
   __shared__ double s_sum[3];
-  if (!reduce_last_block_fast<D::nd>(acc, partials, &ctl->counter, s_sum)) return;
+  if (!reduce_last_block_wide<D::nd>(acc, partials, &ctl->counter, s_sum)) return;
   if (threadIdx.x != 0) return;
   base_apply_scalars<MODE>(ctl, i, slots, s_sum[0], s_sum[1], s_sum[2]);
 }
 
-// Stencil operators: the same step on the tiled z-marching walk (s = A p and
-// the dots in its epilogue, r prefetched one plane ahead where it is read).
+// Stencil operators, pinned order: the same step on the tiled z-marching walk (s =
+// A p and the dots in its epilogue, r prefetched one plane ahead where it is read).
 template <int MODE>
 struct BaseApplyEpi {
   using D = ApplyDots<MODE>;
@@ -250,6 +329,10 @@ struct BaseApplyEpi {
   }
 };
 
+// Planes per work unit, and with them the order of the sums, are chosen for this
+// many resident blocks per SM, not for what a build's registers allow.
+constexpr int kWalkBlocksPerSm = 2;
+
 template <bool ADV, int MODE>
 __global__ void __launch_bounds__(kTileThreads) base_apply_dots_walk(TiledStencil<double, double> T,
                                                                      double* __restrict__ P, double* __restrict__ S,
@@ -264,12 +347,12 @@ __global__ void __launch_bounds__(kTileThreads) base_apply_dots_walk(TiledStenci
   BaseApplyEpi<MODE> e{S + off, r, {}};
   tiled_stencil_walk<double, double, ADV, 1>(T, P + off, e);
   __shared__ double s_sum[3];
-  if (!reduce_last_block_fast<ND>(e.acc, partials, &ctl->counter, s_sum)) return;
+  if (!reduce_last_block_wide<ND>(e.acc, partials, &ctl->counter, s_sum)) return;
   if (threadIdx.x != 0) return;
   base_apply_scalars<MODE>(ctl, i, slots, s_sum[0], s_sum[1], s_sum[2]);
 }
 
-// The same on the flat rows (ncu, 101x97x93, FCG's eta: 44.8 -> 20.4 us, of which the
+// The same on the flat rows, in their order (ncu, 101x97x93, FCG's eta: 44.8 -> 20.4 us, of which the
 // dots no longer formed are a third).
 template <bool ADV, int MODE>
 __global__ void __launch_bounds__(kThreads) base_apply_dots_flat(FlatStencil A, double* __restrict__ P,
@@ -297,8 +380,23 @@ __global__ void __launch_bounds__(kThreads) base_apply_dots_flat(FlatStencil A, 
 
 static int base_template(int mmax) { return mmax <= 8 ? 8 : mmax <= 16 ? 16 : 32; }
 
+static int pinned_dots_blocks(const SolveEnv& env) {
+  const int64_t need = (env.N + kPinThreads - 1) / kPinThreads, cap = (int64_t)env.ctx->num_sms * kPinBlocksPerSm;
+  return (int)(need < cap ? need : cap);
+}
+
 static cudaError_t launch_window_dots(const SolveEnv& env, int tmpl, const double* v, const double* r,
                                       const double* S, int mode) {
+  if (env.pcc.pinned) {
+    const int blocks = pinned_dots_blocks(env);
+    if (!env.partials_fit_2l(blocks, tmpl + 2)) return cudaErrorInvalidValue;
+    switch (tmpl) {
+      case 8: base_window_dots_pinned<8><<<blocks, kPinThreads, 0, env.st>>>(v, r, S, env.N, env.ctl, env.partials, mode); break;
+      case 16: base_window_dots_pinned<16><<<blocks, kPinThreads, 0, env.st>>>(v, r, S, env.N, env.ctl, env.partials, mode); break;
+      default: base_window_dots_pinned<32><<<blocks, kPinThreads, 0, env.st>>>(v, r, S, env.N, env.ctl, env.partials, mode); break;
+    }
+    return cudaGetLastError();
+  }
   const int blocks = window_dots_blocks(env.ctx, env.N);
   if (!env.partials_fit_2l(blocks, tmpl + 2)) return cudaErrorInvalidValue;
   switch (tmpl) {
@@ -323,7 +421,7 @@ template <int MODE>
 static cudaError_t launch_apply_dots(const SolveEnv& env, double* P, double* S, const double* r) {
   const pfk_operator* op = env.op;
   constexpr int ND = ApplyDots<MODE>::nd;
-  if (!op->rowptr && flat_stencil_fits(op)) {
+  if (!op->rowptr && !env.pcc.pinned && flat_stencil_fits(op)) {
     const FlatStencil F = flat_stencil(op);
     const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
     const int blocks = stream_blocks(env.ctx, env.N, 4);
@@ -335,8 +433,7 @@ static cudaError_t launch_apply_dots(const SolveEnv& env, double* P, double* S, 
   if (!op->rowptr) {
     TiledStencil<double, double> T;
     const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
-    const int slots = adv ? tiled_stencil_slots(base_apply_dots_walk<true, MODE>, env.ctx->num_sms)
-                          : tiled_stencil_slots(base_apply_dots_walk<false, MODE>, env.ctx->num_sms);
+    const int slots = kWalkBlocksPerSm * env.ctx->num_sms;
     const int units = tiled_stencil_setup<double, double>(T, op, op->d, op->kx, op->ky, op->kz, slots);
     const int64_t cap = env.partials_cap / ND;
     const int blocks = (int)(units < cap ? units : cap);
@@ -600,6 +697,35 @@ __global__ void __launch_bounds__(kWinThreads, kWinBlocksPerSm) fgb_dots(const d
   if ((int)threadIdx.x < nk) gs->H[threadIdx.x * kGm + gs->k] = s_sum[threadIdx.x];
 }
 
+template <int NW>
+__global__ void __launch_bounds__(kPinThreads, kPinBlocksPerSm) fgb_dots_pinned(const double* __restrict__ z,
+                                                                                const double* __restrict__ P,
+                                                                                int64_t N, SolveCtl* ctl, FgState* gs,
+                                                                                double* partials) {
+  if (ctl->status != kRun) return;
+  constexpr int NWARPS = kPinThreads / 32;
+  __shared__ size_t s_off[NW];
+  __shared__ double s_red[NWARPS * NW];
+  __shared__ double s_sum[NW];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nk = gs->k + 1;           // p_0 .. p_k
+  if (threadIdx.x < nk) s_off[threadIdx.x] = (size_t)threadIdx.x * (size_t)N;
+  __syncthreads();
+  const double gw = window_dots_pinned<NW>(z, P, s_off, nk, N, [](int64_t, double) {});
+  if (lane < nk) s_red[warp * nk + lane] = gw;
+  __syncthreads();
+  if (!combine_block_partials_2l(s_red, nk, partials, NW, &ctl->counter, ctl->gcounter, s_sum)) return;
+  if ((int)threadIdx.x < nk) gs->H[threadIdx.x * kGm + gs->k] = s_sum[threadIdx.x];
+}
+
+template <int NW>
+static void launch_fgb_dots(const SolveEnv& env, const double* z, const double* P, FgState* gs, int blocks) {
+  if (env.pcc.pinned)
+    fgb_dots_pinned<NW><<<blocks, kPinThreads, 0, env.st>>>(z, P, env.N, env.ctl, gs, env.partials);
+  else
+    fgb_dots<NW><<<blocks, kWinThreads, 0, env.st>>>(z, P, env.N, env.ctl, gs, env.partials);
+}
+
 // pbar = z_k - sum_j h_{j,k} p_j into slot k+1, and ||pbar||^2; the last block
 // finishes column k: h_{k+1,k}, Givens, estimate, status.
 template <int NW>
@@ -724,22 +850,22 @@ class Fgmres : public Method {
     (void)x;
     const int* status = &env.ctl->status;
     const int tmpl = base_template(m_ + 1);
-    const int dblocks = window_dots_blocks(env.ctx, N_);
+    const int dblocks = env.pcc.pinned ? pinned_dots_blocks(env) : window_dots_blocks(env.ctx, N_);
     const int oblocks = stream_blocks(env.ctx, N_, 2);
     if (!env.partials_fit_2l(dblocks, tmpl) || !env.partials_fit(oblocks, 1)) return cudaErrorInvalidValue;
     cudaError_t e;
     if ((e = env.mark_pass(0)) != cudaSuccess) return e;
     switch (tmpl) {
       case 8:
-        fgb_dots<8><<<dblocks, kWinThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, env.partials);
+        launch_fgb_dots<8>(env, z_, P_, gs_, dblocks);
         fgb_orth<8><<<oblocks, kThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, m_, env.partials);
         break;
       case 16:
-        fgb_dots<16><<<dblocks, kWinThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, env.partials);
+        launch_fgb_dots<16>(env, z_, P_, gs_, dblocks);
         fgb_orth<16><<<oblocks, kThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, m_, env.partials);
         break;
       default:
-        fgb_dots<32><<<dblocks, kWinThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, env.partials);
+        launch_fgb_dots<32>(env, z_, P_, gs_, dblocks);
         fgb_orth<32><<<oblocks, kThreads, 0, env.st>>>(z_, P_, N_, env.ctl, gs_, m_, env.partials);
         break;
     }

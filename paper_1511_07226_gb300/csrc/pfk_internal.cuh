@@ -282,11 +282,12 @@ __device__ __forceinline__ void block_sums(const double (&acc)[ND], double (&buf
 // w + nwarps, ... (a coalesced row per load, eight rows per step).  Each
 // thread adds its rows in increasing order, then a fixed shuffle tree (nd <=
 // 4) or the warps in order combine them: the sums are deterministic.  smem
-// holds nwarps * nd doubles; out may be shared or global memory.
+// holds nwarps * nd doubles; out may be shared or global memory.  wide: the
+// order of more than four values for any nd.
 __device__ __forceinline__ void sum_rows(const double* rows, int nrows, int nd, int stride, double* smem,
-                                         double* out) {
+                                         double* out, bool wide = false) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  if (nd <= 4) {
+  if (nd <= 4 && !wide) {
     const int T = blockDim.x;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     int b = threadIdx.x;
@@ -469,6 +470,18 @@ __device__ __forceinline__ bool reduce_last_block_fast(const double (&acc)[ND], 
   }
   block_sums<ND>(t, buf, [&](int j, double v) { sums[j] = v; });
   __syncthreads();
+  if (threadIdx.x == 0) *counter = 0u;
+  return true;
+}
+
+// The same with the rows combined in the order of more than four values.
+template <int ND>
+__device__ __forceinline__ bool reduce_last_block_wide(const double (&acc)[ND], double* partials,
+                                                       unsigned int* counter, double* sums) {
+  __shared__ double buf[ND][kThreads];
+  block_sums<ND>(acc, buf, [&](int j, double v) { partials[(size_t)blockIdx.x * ND + j] = v; });
+  if (!arrive_last(counter, gridDim.x)) return false;
+  sum_rows(partials, gridDim.x, ND, ND, &buf[0][0], sums, true);
   if (threadIdx.x == 0) *counter = 0u;
   return true;
 }

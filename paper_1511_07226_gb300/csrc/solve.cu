@@ -217,7 +217,8 @@ pfk_status run_solve(pfk_context* ctx, const pfk_operator* op, const pfk_pc* pc,
   env.partials_cap = pd;
   env.N = N;
   env.pass_ev0 = env.pass_ev1 = nullptr;
-  env.pcc = PcCall{!M->blocking(), h.bar_timeout_ns, &ctx->pinned->pc_gave_up};
+  const bool fp64 = !pc || (pc->kind != PFK_PC_BLOCK_UPPER && pc->precision == PFK_FP64);
+  env.pcc = PcCall{!(M->blocking() && fp64), h.bar_timeout_ns, &ctx->pinned->pc_gave_up};
 
   long long kernel_launches = 0;
 

@@ -3,8 +3,10 @@
 The pipelined recurrences (PIPEFCG, PIPEGCR, PIPEFGMRES and their variants)
 never form a residual or a preconditioned residual anew, so a last-bit
 difference of one inner product grows within some tens of iterations: 26^3
-PIPEGCR at contrast 1e3 moves by up to 5e-7 in 20.  The order in which their
-kernels add is therefore part of their results.  Inputs are exact (integers and
+PIPEGCR at contrast 1e3 moves by up to 5e-7 in 20.  With a preconditioner that
+rounds its input to FP32 the blocking methods' iterates move too, by up to the
+FP32 rounding.  The order in which these kernels add is therefore part of
+their results.  Inputs are exact (integers and
 powers of two): the same bits wherever they are made.
 
 `python tests/_fixed_order.py OUT.json` (repository root as the working folder, a
@@ -58,6 +60,17 @@ CASES = {
     "csr_16": _c("csr", "pipefcg", (64, 64, 1), 16, 24, pc="jacobi", storage="csr"),
     "csr_30": _c("csr", "pipefcg", (64, 64, 1), 30, 48, pc="jacobi", storage="csr"),
     "csr_32": _c("csr", "pipefcg", (125, 139, 1), 32, 40, pc="none", storage="csr"),
+    # FCG, GCR and FGMRES with a preconditioner in reduced precision
+    "prec_fcg": _c("prec", "fcg", (64, 60, 44), 30, 34, precision="fp32"),
+    "prec_fcg_150": _c("prec", "fcg", (150, 92, 85), 16, 18, precision="bf16"),
+    "prec_fcg_8": _c("prec", "fcg", (33, 35, 37), 8, 12, pc="chebyshev", precision="bf16"),
+    "prec_fcg_csr": _c("prec", "fcg", (48, 40, 36), 30, 16, precision="fp32", storage="csr"),
+    "prec_gcr": _c("prec", "gcr", (64, 60, 44), 32, 34, precision="fp32"),
+    "prec_gcr_adv": _c("prec", "gcr", (48, 40, 36), 12, 16, pc="chebyshev", vel=ADV, precision="bf16"),
+    "prec_gcr_csr": _c("prec", "gcr", (300, 210, 1), 30, 16, precision="fp32", storage="csr"),
+    "prec_fgmres": _c("prec", "fgmres", (118, 112, 127), 25, 25, pc="chebyshev", inner=8, vel=ADV, precision="bf16"),
+    "prec_fgmres_8": _c("prec", "fgmres", (40, 33, 21), 7, 14, precision="fp32"),
+    "prec_fgmres_32": _c("prec", "fgmres", (40, 33, 21), 32, 32, pc="chebyshev", vel=ADV, precision="fp32"),
 }
 
 
@@ -81,7 +94,7 @@ def solve_case(ctx, name):
         xs, infos, _ = pfk.solve_grouped(ctx, ops, [b for _, b in probs], pc_kind=c["pc"], inner_iters=c["inner"],
                                          **prm)
         return [(x, i["iterations"]) for x, i in zip(xs, infos)]
-    pc = pfk.Preconditioner(ctx, ops[0], c["pc"], inner_iters=c["inner"])
+    pc = pfk.Preconditioner(ctx, ops[0], c["pc"], inner_iters=c["inner"], precision=c.get("precision", "fp64"))
     x, info, _ = pfk.solve(ctx, ops[0], pc, probs[0][1], **prm)
     return [(x, info["iterations"])]
 
