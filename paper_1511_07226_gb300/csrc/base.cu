@@ -22,7 +22,8 @@ constexpr int kPinStride = kPinThreads + 1;
 static_assert(kWinBlocksPerSm <= kMaxBlocksPerSm && kPinBlocksPerSm <= kMaxBlocksPerSm,
               "partials are sized for kMaxBlocksPerSm blocks per SM");
 
-// A CSR operator (stencil operators take the tiled walk).
+// A CSR operator (stencil operators take the flat rows, or the tiled walk for
+// sums in a pinned order).
 struct CsrView {
   const int32_t* rowptr;
   const int32_t* colidx;
@@ -352,10 +353,10 @@ __global__ void __launch_bounds__(kTileThreads) base_apply_dots_walk(TiledStenci
   base_apply_scalars<MODE>(ctl, i, slots, s_sum[0], s_sum[1], s_sum[2]);
 }
 
-// The same on the flat rows, in their order (ncu, 101x97x93, FCG's eta: 44.8 -> 20.4 us, of which the
-// dots no longer formed are a third).
-template <bool ADV, int MODE>
-__global__ void __launch_bounds__(kThreads) base_apply_dots_flat(FlatStencil A, double* __restrict__ P,
+// The same on the flat rows, in their order (ncu, 101x97x93, FCG's eta: 44.8 -> 20.4 us,
+// of which the dots no longer formed are a third).
+template <bool ADV, int MODE, typename I>
+__global__ void __launch_bounds__(kThreads) base_apply_dots_flat(FlatStencilT<I> A, double* __restrict__ P,
                                                                  double* __restrict__ S, const double* __restrict__ r,
                                                                  int64_t N, SolveCtl* ctl, double* partials) {
   if (ctl->status != kRun) return;
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(kThreads) base_apply_dots_flat(FlatStencil A, 
   const size_t off = (size_t)(i % slots) * (size_t)N;
   BaseApplyEpi<MODE> e{S + off, r, {}};
   const double* p = P + off;
-  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
+  FLAT_CELLS(I, c, A.n) {
     const auto pre = e.pre(c);
     double pv;
     const double sv = flat_row<ADV>(A, p, c, pv);
@@ -421,13 +422,13 @@ template <int MODE>
 static cudaError_t launch_apply_dots(const SolveEnv& env, double* P, double* S, const double* r) {
   const pfk_operator* op = env.op;
   constexpr int ND = ApplyDots<MODE>::nd;
-  if (!op->rowptr && !env.pcc.pinned && flat_stencil_fits(op)) {
-    const FlatStencil F = flat_stencil(op);
-    const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
+  if (!op->rowptr && !env.pcc.pinned) {
     const int blocks = stream_blocks(env.ctx, env.N, 4);
     if (!env.partials_fit(blocks, ND)) return cudaErrorInvalidValue;
-    if (adv) base_apply_dots_flat<true, MODE><<<blocks, kThreads, 0, env.st>>>(F, P, S, r, env.N, env.ctl, env.partials);
-    else base_apply_dots_flat<false, MODE><<<blocks, kThreads, 0, env.st>>>(F, P, S, r, env.N, env.ctl, env.partials);
+    with_flat_stencil(op, [&](const auto& A, auto adv) {
+      base_apply_dots_flat<adv.value, MODE><<<blocks, kThreads, 0, env.st>>>(A, P, S, r, env.N, env.ctl,
+                                                                             env.partials);
+    });
     return cudaGetLastError();
   }
   if (!op->rowptr) {
@@ -613,35 +614,14 @@ __global__ void __launch_bounds__(kThreads) fgb_apply_store(CsrView A, const dou
   }
 }
 
-// Stencil operators: z = A u and the copy of u into U on the tiled walk.
-struct FgStoreEpi {
-  double* __restrict__ z;
-  double* __restrict__ u;
-  struct Pre {};
-  __device__ __forceinline__ Pre pre(int64_t) const { return Pre{}; }
-  __device__ __forceinline__ void operator()(int64_t c, double zv, double uv, const Pre&) const {
-    z[c] = zv;
-    u[c] = uv;
-  }
-};
-
-template <bool ADV>
-__global__ void __launch_bounds__(kTileThreads) fgb_apply_store_walk(TiledStencil<double, double> T,
-                                                                     const double* __restrict__ ucur,
-                                                                     double* __restrict__ U, double* __restrict__ z,
-                                                                     int64_t N, const FgState* gs, const int* status) {
-  if (*status != kRun) return;
-  FgStoreEpi e{z, U + (size_t)gs->k * (size_t)N};
-  tiled_stencil_walk<double, double, ADV, 1>(T, ucur, e);
-}
-
-template <bool ADV>
-__global__ void __launch_bounds__(kThreads) fgb_apply_store_flat(FlatStencil A, const double* __restrict__ ucur,
+// The same for stencil operators.
+template <bool ADV, typename I>
+__global__ void __launch_bounds__(kThreads) fgb_apply_store_flat(FlatStencilT<I> A, const double* __restrict__ ucur,
                                                                  double* __restrict__ U, double* __restrict__ z,
                                                                  int64_t N, const FgState* gs, const int* status) {
   if (*status != kRun) return;
   double* u = U + (size_t)gs->k * (size_t)N;
-  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
+  FLAT_CELLS(I, c, A.n) {
     double uv;
     z[c] = flat_row<ADV>(A, ucur, c, uv);
     u[c] = uv;
@@ -651,24 +631,13 @@ __global__ void __launch_bounds__(kThreads) fgb_apply_store_flat(FlatStencil A, 
 static cudaError_t launch_apply_store(const SolveEnv& env, const double* ucur, double* U, double* z,
                                       const FgState* gs, const int* status) {
   const pfk_operator* op = env.op;
-  if (!op->rowptr && flat_stencil_fits(op)) {
-    const FlatStencil F = flat_stencil(op);
-    const int blocks = stream_blocks(env.ctx, env.N, 8);
-    if (op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0)
-      fgb_apply_store_flat<true><<<blocks, kThreads, 0, env.st>>>(F, ucur, U, z, env.N, gs, status);
-    else
-      fgb_apply_store_flat<false><<<blocks, kThreads, 0, env.st>>>(F, ucur, U, z, env.N, gs, status);
-  } else if (!op->rowptr) {
-    TiledStencil<double, double> T;
-    const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
-    const int slots = adv ? tiled_stencil_slots(fgb_apply_store_walk<true>, env.ctx->num_sms)
-                          : tiled_stencil_slots(fgb_apply_store_walk<false>, env.ctx->num_sms);
-    const int units = tiled_stencil_setup<double, double>(T, op, op->d, op->kx, op->ky, op->kz, slots);
-    if (adv) fgb_apply_store_walk<true><<<units, kTileThreads, 0, env.st>>>(T, ucur, U, z, env.N, gs, status);
-    else fgb_apply_store_walk<false><<<units, kTileThreads, 0, env.st>>>(T, ucur, U, z, env.N, gs, status);
+  const int blocks = stream_blocks(env.ctx, env.N, 8);
+  if (op->rowptr) {
+    fgb_apply_store<<<blocks, kThreads, 0, env.st>>>(csr_of(op), ucur, U, z, env.N, gs, status);
   } else {
-    fgb_apply_store<<<stream_blocks(env.ctx, env.N, 8), kThreads, 0, env.st>>>(csr_of(op), ucur, U, z, env.N, gs,
-                                                                               status);
+    with_flat_stencil(op, [&](const auto& A, auto adv) {
+      fgb_apply_store_flat<adv.value><<<blocks, kThreads, 0, env.st>>>(A, ucur, U, z, env.N, gs, status);
+    });
   }
   return cudaGetLastError();
 }

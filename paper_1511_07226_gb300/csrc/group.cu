@@ -113,7 +113,7 @@ struct GrpSys {
   int u0, u1, u2;
   int adv;            // any advection weight non-zero
   int nblk;           // CTAs of the group
-  int sx, sy;         // c / nx = (c mx) >> sx, row / ny = (row my) >> sy for c < 2^31 (mx = 0: larger system)
+  int sx, sy;         // c / nx = (c mx) >> sx, row / ny = (row my) >> sy
   unsigned mx, my;
   int pad0;
   const double* b;
@@ -259,10 +259,10 @@ __device__ void grp_sum(const GrpSys& S, GrpCta* g, const double (&v)[ND], doubl
 // whatever the row length -- an FP64 instruction holds the pipe as long with a
 // few active lanes as with 32, and a row per warp leaves 24 of 64 lanes idle at
 // nx = 40.  Otherwise a row per warp (the order the FP32 inner products were
-// pinned with, and systems of 2^31 cells or more).
+// pinned with).
 template <bool FLAT, typename F>
 __device__ __forceinline__ void grp_cells(const GrpSys& S, const GrpCta* g, F&& f) {
-  if (FLAT && S.mx) {
+  if constexpr (FLAT) {
     const unsigned nx = (unsigned)S.nx, ny = (unsigned)S.ny;
     const unsigned end = (unsigned)(g->row_hi * S.nx);
     const unsigned beg = (unsigned)(g->row_lo * S.nx);
@@ -1512,12 +1512,8 @@ pfk_status GroupRunner::admit(const pfk_operator* op, const pfk_pc_desc* pcd, co
   S.u0 = op->upw[0]; S.u1 = op->upw[1]; S.u2 = op->upw[2];
   S.adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
   S.nblk = nblk;
-  S.mx = S.my = 0u;
-  S.sx = S.sy = 0;
-  if (flat_stencil_fits(op)) {
-    const FlatStencil F = flat_stencil(op);
-    S.mx = F.mx; S.my = F.my; S.sx = F.sx; S.sy = F.sy;
-  }
+  const FlatStencilT<unsigned> F = flat_stencil<unsigned>(op);   // (an eligible system has at most INT32_MAX cells)
+  S.mx = F.mx; S.my = F.my; S.sx = F.sx; S.sy = F.sy;
   S.b = b_dev;
   S.x = x_dev;
   S.ws = (double*)mem;

@@ -6,7 +6,6 @@
 // performance model (Sec. 8): the T_spmv term of every method.  It is the
 // "A" of every listing (Algs. 2-15).
 #include "pfk_internal.cuh"
-#include "stencil.cuh"
 #include "stencil_flat.cuh"
 
 #include <cmath>
@@ -136,38 +135,14 @@ struct StencilArgs {
   int64_t n;
 };
 
-// y = A m (or bsub - A m) with the tiled z-marching walk.
-struct ApplyEpi {
-  double* __restrict__ y;
-  const double* __restrict__ bsub;
-  struct Pre {
-    double b;
-  };
-  __device__ __forceinline__ Pre pre(int64_t c) const { return Pre{bsub ? bsub[c] : 0.0}; }
-  __device__ __forceinline__ void operator()(int64_t c, double v, double, const Pre& p) const {
-    y[c] = bsub ? p.b - v : v;
-  }
-};
-
-template <bool ADV>
-__global__ void __launch_bounds__(kTileThreads) stencil_tiled_apply_kernel(TiledStencil<double, double> A,
-                                                                           const double* __restrict__ m,
-                                                                           double* __restrict__ y,
-                                                                           const double* __restrict__ bsub,
-                                                                           const int* __restrict__ status) {
+// y = A m, or bsub - A m.
+template <bool ADV, typename I>
+__global__ void __launch_bounds__(kThreads) stencil_apply_kernel(FlatStencilT<I> A, const double* __restrict__ m,
+                                                                 double* __restrict__ y,
+                                                                 const double* __restrict__ bsub,
+                                                                 const int* __restrict__ status) {
   if (status && *status != kRun) return;
-  ApplyEpi e{y, bsub};
-  tiled_stencil_walk<double, double, ADV, 1>(A, m, e);
-}
-
-// The same on the flat form.
-template <bool ADV>
-__global__ void __launch_bounds__(kThreads) stencil_flat_apply_kernel(FlatStencil A, const double* __restrict__ m,
-                                                                      double* __restrict__ y,
-                                                                      const double* __restrict__ bsub,
-                                                                      const int* __restrict__ status) {
-  if (status && *status != kRun) return;
-  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
+  FLAT_CELLS(I, c, A.n) {
     double mc;
     const double v = flat_row<ADV>(A, m, c, mc);
     y[c] = bsub ? bsub[c] - v : v;
@@ -270,20 +245,10 @@ cudaError_t op_apply(const pfk_operator* op, const double* x, double* y, const d
   const int blocks = stream_blocks(op->ctx, op->n, 8);
   if (op->rowptr) {
     csr_apply_kernel<<<blocks, kThreads, 0, st>>>(op->rowptr, op->colidx, op->vals, x, y, bsub, op->n, status);
-  } else if (flat_stencil_fits(op)) {
-    const FlatStencil A = flat_stencil(op);
-    if (op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0)
-      stencil_flat_apply_kernel<true><<<blocks, kThreads, 0, st>>>(A, x, y, bsub, status);
-    else
-      stencil_flat_apply_kernel<false><<<blocks, kThreads, 0, st>>>(A, x, y, bsub, status);
   } else {
-    TiledStencil<double, double> A;
-    const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
-    const int slots = adv ? tiled_stencil_slots(stencil_tiled_apply_kernel<true>, op->ctx->num_sms)
-                          : tiled_stencil_slots(stencil_tiled_apply_kernel<false>, op->ctx->num_sms);
-    const int units = tiled_stencil_setup<double, double>(A, op, op->d, op->kx, op->ky, op->kz, slots);
-    if (adv) stencil_tiled_apply_kernel<true><<<units, kTileThreads, 0, st>>>(A, x, y, bsub, status);
-    else stencil_tiled_apply_kernel<false><<<units, kTileThreads, 0, st>>>(A, x, y, bsub, status);
+    with_flat_stencil(op, [&](const auto& A, auto adv) {
+      stencil_apply_kernel<adv.value><<<blocks, kThreads, 0, st>>>(A, x, y, bsub, status);
+    });
   }
   return cudaGetLastError();
 }

@@ -289,14 +289,14 @@ __device__ __forceinline__ void pcg_c_scalars(PcCtl* ctl, int i, double eta) {
 }
 
 // FP64 C_i on the flat rows (ncu: 128^3 42.7 -> 36.1 us, 150x141x133 55.4 -> 47.3 us).
-template <bool ADV>
-__global__ void __launch_bounds__(kThreads) pcg_c_flat_kernel(FlatStencil A, const double* __restrict__ p,
+template <bool ADV, typename I>
+__global__ void __launch_bounds__(kThreads) pcg_c_flat_kernel(FlatStencilT<I> A, const double* __restrict__ p,
                                                               double* __restrict__ s, PcCtl* ctl, int i,
                                                               double* partials, const int* __restrict__ status) {
   const int run = status ? *status : (int)kRun, ok = ctl->ok;
   if (run != kRun || !(i < ok)) return;
   double acc[1] = {0.0};
-  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
+  FLAT_CELLS(I, c, A.n) {
     double pv;
     const double sv = flat_row<ADV>(A, p, c, pv);
     s[c] = sv;
@@ -396,15 +396,15 @@ __global__ void __launch_bounds__(kTileThreads, 3) cheb_sweep_kernel(TiledStenci
   tiled_stencil_walk<V, C, ADV, tiled_width<V, C>()>(T, dj, e);
 }
 
-// The FP64 sweep on the flat rows (same results).
-template <bool ADV>
-__global__ void __launch_bounds__(kThreads) cheb_flat_kernel(FlatStencil A, const double* __restrict__ dinv,
+// The FP64 sweep: the same on the flat rows.
+template <bool ADV, typename I>
+__global__ void __launch_bounds__(kThreads) cheb_flat_kernel(FlatStencilT<I> A, const double* __restrict__ dinv,
                                                              const double* __restrict__ dj, double* __restrict__ dn,
                                                              double* __restrict__ r, double* __restrict__ x, int j,
                                                              double c1, double c2, const int* __restrict__ status) {
   SKIP_IF_DONE(status);
   ChebEpi<double, double> e{dinv, dn, r, x, j == 0, c1, c2};
-  for (unsigned c = blockIdx.x * kThreads + threadIdx.x; c < A.n; c += gridDim.x * kThreads) {
+  FLAT_CELLS(I, c, A.n) {
     const auto pre = e.pre(c);
     double dc;
     const double ad = flat_row<ADV>(A, dj, c, dc);
@@ -599,10 +599,10 @@ static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v
       }
     }
     if constexpr (F64) {
-      if (!pinned && flat_stencil_fits(op)) {
-        const FlatStencil F = flat_stencil(op);
-        if (T.adv) pcg_c_flat_kernel<true><<<blocks, kThreads, 0, st>>>(F, pv, s, ctl, i, pc->partials, status);
-        else pcg_c_flat_kernel<false><<<blocks, kThreads, 0, st>>>(F, pv, s, ctl, i, pc->partials, status);
+      if (!pinned) {
+        with_flat_stencil(op, [&](const auto& F, auto adv) {
+          pcg_c_flat_kernel<adv.value><<<blocks, kThreads, 0, st>>>(F, pv, s, ctl, i, pc->partials, status);
+        });
         return;
       }
     }
@@ -632,16 +632,17 @@ static cudaError_t chebyshev(const pfk_pc* pc, StencilT<V, C> A, const double* v
   const double theta = (pc->hi + pc->lo) / 2.0, delta = (pc->hi - pc->lo) / 2.0;
   const double sigma1 = theta / delta;
   double rho = 1.0 / sigma1;
-  TiledStencil<V, C> T;
   const pfk_operator* op = pc->op;
-  const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
-  const int slots = adv ? tiled_stencil_slots(cheb_sweep_kernel<V, C, true>, pc->ctx->num_sms)
-                        : tiled_stencil_slots(cheb_sweep_kernel<V, C, false>, pc->ctx->num_sms);
-  const int units = tiled_stencil_setup<V, C>(T, op, A.d, A.kx, A.ky, A.kz, slots);
-  // reduced precision on an aligned 3-D grid: the TMA-pipelined walk
+  // reduced precision: the tiled walk, TMA-pipelined on an aligned 3-D grid
+  TiledStencil<V, C> T;
+  int units = 0;
   bool tma = false;
   TmaMaps maps[2];
   if constexpr (std::is_same<V, float>::value) {
+    const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
+    const int slots = adv ? tiled_stencil_slots(cheb_sweep_kernel<V, C, true>, pc->ctx->num_sms)
+                          : tiled_stencil_slots(cheb_sweep_kernel<V, C, false>, pc->ctx->num_sms);
+    units = tiled_stencil_setup<V, C>(T, op, A.d, A.kx, A.ky, A.kz, slots);
     tma = tma_walk_usable(op->nx, op->nz, {dv[0], dv[1], r, x, A.d, A.kx, A.ky, A.kz, A.dinv}) &&
           tma_maps<C>(maps[0], op, dv[0], A.d, A.kx, A.ky, A.kz, A.dinv, r, x) &&
           tma_maps<C>(maps[1], op, dv[1], A.d, A.kx, A.ky, A.kz, A.dinv, r, x);
@@ -650,41 +651,29 @@ static cudaError_t chebyshev(const pfk_pc* pc, StencilT<V, C> A, const double* v
   for (int j = 0; j + 1 < k; ++j) {
     const double rho_new = 1.0 / (2.0 * sigma1 - rho);
     const V c1 = (V)(rho_new * rho), c2 = (V)(2.0 * rho_new / delta);
-    if constexpr (std::is_same<V, float>::value) {
-      if (tma) {
-        TmaWalkArgs a{};
-        a.dn = dv[(j + 1) & 1];
-        a.r = r;
-        a.x = x;
-        a.first = j == 0;
-        a.c1 = c1;
-        a.c2 = c2;
-        a.status = status;
-        a.err = (int*)pc->ctx->scratch_counter + 3;
-        tma_launch<C, true>(maps[j & 1], a, op, st);
-        rho = rho_new;
-        continue;
-      }
-    }
     if constexpr (std::is_same<V, double>::value) {
-      if (flat_stencil_fits(op)) {
-        const FlatStencil F = flat_stencil(op);
-        if (T.adv)
-          cheb_flat_kernel<true><<<sblocks, kThreads, 0, st>>>(F, A.dinv, dv[j & 1], dv[(j + 1) & 1], r, x, j, c1, c2,
-                                                               status);
-        else
-          cheb_flat_kernel<false><<<sblocks, kThreads, 0, st>>>(F, A.dinv, dv[j & 1], dv[(j + 1) & 1], r, x, j, c1, c2,
-                                                                status);
-        rho = rho_new;
-        continue;
-      }
-    }
-    if (T.adv)
+      with_flat_stencil(op, [&](const auto& F, auto adv) {
+        cheb_flat_kernel<adv.value><<<sblocks, kThreads, 0, st>>>(F, A.dinv, dv[j & 1], dv[(j + 1) & 1], r, x, j, c1,
+                                                                  c2, status);
+      });
+    } else if (tma) {
+      TmaWalkArgs a{};
+      a.dn = dv[(j + 1) & 1];
+      a.r = r;
+      a.x = x;
+      a.first = j == 0;
+      a.c1 = c1;
+      a.c2 = c2;
+      a.status = status;
+      a.err = (int*)pc->ctx->scratch_counter + 3;
+      tma_launch<C, true>(maps[j & 1], a, op, st);
+    } else if (T.adv) {
       cheb_sweep_kernel<V, C, true><<<units, kTileThreads, 0, st>>>(T, A.dinv, dv[j & 1], dv[(j + 1) & 1], r, x, j,
                                                                     c1, c2, status);
-    else
+    } else {
       cheb_sweep_kernel<V, C, false><<<units, kTileThreads, 0, st>>>(T, A.dinv, dv[j & 1], dv[(j + 1) & 1], r, x, j,
                                                                      c1, c2, status);
+    }
     rho = rho_new;
   }
   cheb_last_kernel<V><<<sblocks, kThreads, 0, st>>>(n, dv[(k - 1) & 1], x, k == 1, add, out, status);

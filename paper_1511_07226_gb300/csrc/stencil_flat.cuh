@@ -8,36 +8,40 @@
 // Here a warp takes 32 consecutive cells of the whole grid, so no lane idles
 // whatever the sides, and there is no barrier: the neighbours come through L1
 // and L2 (11 values of 8 bytes per cell cross L2, 5.8 TB/s at the FP64 rate).
-// The terms are added in the walk's order: the same result bit for bit.
-// Operator application, walk -> flat rows: 256^3 with advection 269 -> 233 us
-// (FP64 instruction floor 222), 200 x 199 x 198 156 -> 119, 101 x 97 x 93 41 ->
-// 31, 2048 x 1500 83 -> 47, 64^3 26 -> 22.
+// The terms are added in the walk's order: the same result bit for bit.  Operator
+// application, walk -> flat rows: 256^3 269 -> 233 us (FP64 instruction floor 222),
+// 200 x 199 x 198 156 -> 119, 101 x 97 x 93 41 -> 31, 2048 x 1500 83 -> 47, 64^3
+// 26 -> 22; 256^3 with advection 365 either way (floor 317).  Never slower, so
+// every FP64 stencil without a sum in a pinned order takes them.
 #pragma once
 
 #include "pfk_internal.cuh"
 
+#include <type_traits>
+
 namespace pfk {
 
-struct FlatStencil {
+// I: the type of a cell index, unsigned below 2^31 cells (a row and a plane by
+// multiply and shift), else unsigned long long (by division).
+template <typename I>
+struct FlatStencilT {
   const double* d;
   const double* kx;
   const double* ky;
   const double* kz;
-  unsigned nx, ny, nz, n;
+  unsigned nx, ny, nz;
+  I n;
   unsigned mx, my;      // c / nx = (c mx) >> sx for c < 2^31
   int sx, sy;
   double a0, a1, a2;    // upwind weights h |v_d|
   int up0, up1, up2;    // side of the upwind neighbour: -1 (v_d > 0) or +1
 };
 
-// The flat rows are faster at every measured size (figures above), so only the
-// 31-bit cell count limits them; larger grids take the tiled walk.
-inline bool flat_stencil_fits(const pfk_operator* op) { return op->n < (int64_t)1 << 31; }
-
-inline FlatStencil flat_stencil(const pfk_operator* op) {
-  FlatStencil A;
+template <typename I>
+inline FlatStencilT<I> flat_stencil(const pfk_operator* op) {
+  FlatStencilT<I> A;
   A.d = op->d; A.kx = op->kx; A.ky = op->ky; A.kz = op->kz;
-  A.nx = (unsigned)op->nx; A.ny = (unsigned)op->ny; A.nz = (unsigned)op->nz; A.n = (unsigned)op->n;
+  A.nx = (unsigned)op->nx; A.ny = (unsigned)op->ny; A.nz = (unsigned)op->nz; A.n = (I)op->n;
   auto magic = [](unsigned dv, unsigned& m, int& s) {   // m = ceil(2^(31 + l) / dv), l = ceil(log2 dv): exact below 2^31
     int l = 0;
     while ((1ull << l) < dv) ++l;
@@ -53,13 +57,36 @@ inline FlatStencil flat_stencil(const pfk_operator* op) {
   return A;
 }
 
+// Host: f(stencil, bool_constant<advection>) with the index type and the
+// advection form of the operator.
+template <typename F>
+inline void with_flat_stencil(const pfk_operator* op, F&& f) {
+  const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
+  auto go = [&](const auto& A) {
+    if (adv) f(A, std::true_type{});
+    else f(A, std::false_type{});
+  };
+  if (op->n < (int64_t)1 << 31) go(flat_stencil<unsigned>(op));
+  else go(flat_stencil<unsigned long long>(op));
+}
+
+// The cells of a grid-stride loop.
+#define FLAT_CELLS(I, c, n) \
+  for (I c = blockIdx.x * (I)kThreads + threadIdx.x; c < (n); c += gridDim.x * (I)kThreads)
+
 // (A m)_c; mc = m[c].
-template <bool ADV>
-__device__ __forceinline__ double flat_row(const FlatStencil& A, const double* __restrict__ m, unsigned c,
-                                           double& mc) {
-  const unsigned row = (unsigned)(((unsigned long long)c * A.mx) >> A.sx), i = c - row * A.nx;
-  const unsigned k = (unsigned)(((unsigned long long)row * A.my) >> A.sy), j = row - k * A.ny;
-  const unsigned sxy = A.nx * A.ny;
+template <bool ADV, typename I>
+__device__ __forceinline__ double flat_row(const FlatStencilT<I>& A, const double* __restrict__ m, I c, double& mc) {
+  I row, k;
+  if constexpr (sizeof(I) == 4) {
+    row = (unsigned)(((unsigned long long)c * A.mx) >> A.sx);
+    k = (unsigned)(((unsigned long long)row * A.my) >> A.sy);
+  } else {
+    row = c / A.nx;
+    k = row / A.ny;
+  }
+  const unsigned i = (unsigned)(c - row * A.nx), j = (unsigned)(row - k * A.ny);
+  const I sxy = (I)A.nx * A.ny;
   const bool xm = i > 0, xp = i + 1 < A.nx, ym = j > 0, yp = j + 1 < A.ny;
   mc = m[c];
   const double d = A.d[c], kx = A.kx[c], ky = A.ky[c];
