@@ -149,11 +149,16 @@ __device__ __forceinline__ bool pcg_reduce(const double (&acc)[1], double* parti
   }
 }
 
+// Blocks per SM of the inner PCG's reducing kernels, all of them resident at once
+// (8: 32 registers); the grid is part of the order of the sums (inner_pcg).
+template <typename V>
+__host__ __device__ constexpr int pcg_grid_per_sm(bool pinned) { return sizeof(V) == 4 || pinned ? 8 : 4; }
+
 // A_0 and B_0 in one launch (neither needs the other's result):
 // r_0 = v (not stored: A_1 reads v), p_0 = D^-1 r_0, gamma_0 = <D^-1 r_0, r_0>;
 // finalize: stop at once (B(v) = 0) if gamma_0 == 0 (then v and p_0 are zero).
-template <typename V, typename C>
-__global__ void __launch_bounds__(kThreads) pcg_first_kernel(StencilT<V, C> A, const double* __restrict__ v,
+template <typename V, typename C, bool PIN>
+__global__ void __launch_bounds__(kThreads, pcg_grid_per_sm<V>(PIN)) pcg_first_kernel(StencilT<V, C> A, const double* __restrict__ v,
                                                              V* __restrict__ p0, PcCtl* ctl, int k,
                                                              double* partials, const int* __restrict__ status) {
   SKIP_IF_DONE(status);
@@ -179,8 +184,8 @@ __global__ void __launch_bounds__(kThreads) pcg_first_kernel(StencilT<V, C> A, c
 // that B_i reads it instead of r_i and D^-1: one FP64 product and one array less
 // there (both kernels are balanced between the FP64 pipe and HBM).  The control
 // words are loaded together: one L2 round trip instead of three in a row.
-template <typename V, typename C>
-__global__ void __launch_bounds__(kThreads) pcg_a_kernel(StencilT<V, C> A, const double* __restrict__ v,
+template <typename V, typename C, bool PIN>
+__global__ void __launch_bounds__(kThreads, pcg_grid_per_sm<V>(PIN)) pcg_a_kernel(StencilT<V, C> A, const double* __restrict__ v,
                                                          V* __restrict__ r, V* __restrict__ s, PcCtl* ctl,
                                                          int i, double* partials, const int* __restrict__ status) {
   const int run = status ? *status : (int)kRun, last_x = ctl->ok;
@@ -189,8 +194,8 @@ __global__ void __launch_bounds__(kThreads) pcg_a_kernel(StencilT<V, C> A, const
   V accv = V(0);
   const int64_t T = (int64_t)gridDim.x * blockDim.x;
   int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  // FP64: two cells' loads in flight, added in order (half the blocks of the FP32 form)
-  for (; std::is_same<V, double>::value && c + T < A.n; c += 2 * T) {
+  // FP64 at half the blocks: two cells' loads in flight, added in order
+  for (; std::is_same<V, double>::value && !PIN && c + T < A.n; c += 2 * T) {
     const V r0 = i == 1 ? (V)v[c] : r[c], r1 = i == 1 ? (V)v[c + T] : r[c + T];
     const V s0 = s[c], s1 = s[c + T];
     const V d0 = cv<V, C>(A.dinv[c]), d1 = cv<V, C>(A.dinv[c + T]);
@@ -564,8 +569,7 @@ static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v
   const int k = pc->inner;
   const int sblocks = stream_blocks(pc->ctx, n, 8);
   const int bblocks = F64 ? stream_blocks(pc->ctx, n, 4) : sblocks;   // B_i: two cells per thread and step
-  // reducing kernels: the grid fixes the order of the sums (FP32: a thread's FP32 partial sums)
-  const int blocks = F64 && !pinned ? bblocks : sblocks;
+  const int blocks = stream_blocks(pc->ctx, n, pcg_grid_per_sm<V>(pinned));   // reducing kernels
   TiledStencil<V, C> T;
   const pfk_operator* op = pc->op;
   const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
@@ -575,7 +579,8 @@ static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v
   const int units = tiled_stencil_setup<V, C>(T, op, A.d, A.kx, A.ky, A.kz, slots);
   const int tblocks = units < pc->partials_cap ? units : pc->partials_cap;
   PcCtl* ctl = pc->ctl;
-  pcg_first_kernel<V, C><<<blocks, kThreads, 0, st>>>(A, v, p[0], ctl, k, pc->partials, status);
+  if (F64 && pinned) pcg_first_kernel<V, C, F64><<<blocks, kThreads, 0, st>>>(A, v, p[0], ctl, k, pc->partials, status);
+  else pcg_first_kernel<V, C, false><<<blocks, kThreads, 0, st>>>(A, v, p[0], ctl, k, pc->partials, status);
   // reduced precision on an aligned 3-D grid: the TMA-pipelined walk
   bool tma = false;
   TmaMaps maps[2];
@@ -611,7 +616,8 @@ static cudaError_t inner_pcg(const pfk_pc* pc, StencilT<V, C> A, const double* v
   };
   pcg_c(p[0], 0);
   for (int i = 1; i < k; ++i) {
-    pcg_a_kernel<V, C><<<blocks, kThreads, 0, st>>>(A, v, r, s, ctl, i, pc->partials, status);
+    if (F64 && pinned) pcg_a_kernel<V, C, F64><<<blocks, kThreads, 0, st>>>(A, v, r, s, ctl, i, pc->partials, status);
+    else pcg_a_kernel<V, C, false><<<blocks, kThreads, 0, st>>>(A, v, r, s, ctl, i, pc->partials, status);
     pcg_b_kernel<V, C><<<bblocks, kThreads, 0, st>>>(A, F64 ? s : r, p[(i - 1) & 1], p[i & 1], x, ctl, i, status);
     pcg_c(p[i & 1], i);
   }
