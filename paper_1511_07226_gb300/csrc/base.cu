@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kThreads) base_apply_dots_flat(FlatStencilT<I>
     e(c, sv, pv, pre);
   }
   __shared__ double s_sum[3];
-  if (!reduce_last_block_fast<ND>(e.acc, partials, &ctl->counter, s_sum)) return;
+  if (!reduce_last_block_fast<ND, true>(e.acc, partials, &ctl->counter, s_sum)) return;
   if (threadIdx.x != 0) return;
   base_apply_scalars<MODE>(ctl, i, slots, s_sum[0], s_sum[1], s_sum[2]);
 }

@@ -14,10 +14,9 @@
 //                (Saad, Iterative Methods for Sparse Linear Systems, 2nd ed.,
 //                Alg. 12.1), one fused kernel per sweep.
 //
-// Precision variants (spec mixed precision): vectors V = double or
-// float, coefficient storage C = double, float or bfloat16.  Inner products of
-// the FP32 variants accumulate per thread in FP32 and are combined across
-// threads and blocks in FP64.
+// Precision variants: vectors V = double or float, coefficient storage C =
+// double, float or bfloat16.  Inner products of the FP32 variants accumulate per
+// thread in FP32 and are combined across threads and blocks in FP64.
 #include "pfk_internal.cuh"
 #include "stencil.cuh"
 #include "stencil_flat.cuh"
@@ -138,11 +137,11 @@ __global__ void __launch_bounds__(kThreads) noisy_row_norms_kernel(const double*
 
 // The reductions of the inner PCG: the FP32 form keeps the order its results
 // were pinned with.
-template <typename V>
+template <typename V, bool FREE>
 __device__ __forceinline__ bool pcg_reduce(const double (&acc)[1], double* partials, unsigned int* counter,
                                            double* sums) {
   if constexpr (std::is_same<V, double>::value) {
-    return reduce_last_block_fast<1>(acc, partials, counter, sums);
+    return reduce_last_block_fast<1, FREE>(acc, partials, counter, sums);
   } else {
     __shared__ double smem[kThreads / 32];
     return reduce_last_block<1>(acc, 1, partials, 1, counter, smem, sums);
@@ -171,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, pcg_grid_per_sm<V>(PIN)) pcg_first_k
   }
   double acc[1] = {(double)accv};
   __shared__ double sums[1];
-  if (pcg_reduce<V>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0) {
+  if (pcg_reduce<V, !PIN>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0) {
     const double g = sums[0];
     ctl->gamma = g;
     ctl->ok = (g == 0.0) ? 0 : k;
@@ -217,7 +216,7 @@ __global__ void __launch_bounds__(kThreads, pcg_grid_per_sm<V>(PIN)) pcg_a_kerne
   }
   double acc[1] = {(double)accv};
   __shared__ double sums[1];
-  if (pcg_reduce<V>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0) {
+  if (pcg_reduce<V, !PIN>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0) {
     const double g = sums[0];
     if (g == 0.0) {
       ctl->ok = i;
@@ -308,7 +307,7 @@ __global__ void __launch_bounds__(kThreads) pcg_c_flat_kernel(FlatStencilT<I> A,
     acc[0] = fma(sv, pv, acc[0]);
   }
   __shared__ double sums[1];
-  if (reduce_last_block_fast<1>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0)
+  if (reduce_last_block_fast<1, true>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0)
     pcg_c_scalars(ctl, i, sums[0]);
 }
 
@@ -322,7 +321,7 @@ __global__ void __launch_bounds__(kTileThreads) pcg_c_kernel(TiledStencil<V, C> 
   tiled_stencil_walk<V, C, ADV, tiled_width<V, C>()>(T, p, e);
   double acc[1] = {(double)e.acc};
   __shared__ double sums[1];
-  if (pcg_reduce<V>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0) pcg_c_scalars(ctl, i, sums[0]);
+  if (pcg_reduce<V, false>(acc, partials, &ctl->counter, sums) && threadIdx.x == 0) pcg_c_scalars(ctl, i, sums[0]);
 }
 
 // F.  x_k = x_{k-1} + alpha_{k-1} p_{k-1} if the loop reached iteration k;

@@ -253,8 +253,11 @@ __device__ __forceinline__ double warp_sum_transposed(double (&acc)[V]) {
 // transposed (9 additions) and adds the eight sums (7), so a value costs the
 // block 16 FP64 instructions instead of 48; the warp rotates with the block
 // so that the resident blocks' sums spread over the SM's four FP64 pipes.
+// FREE: the eight warps' values lane by lane, then one tree, in an order of its
+// own, for sums that are not pinned: 12 instructions and a shorter chain (an
+// application of the separate inner PCG kernels, 150 x 141 x 133: 385 -> 370 us).
 // store(j, sum) is called by lane 0 of that warp.
-template <int ND, typename F>
+template <int ND, bool FREE, typename F>
 __device__ __forceinline__ void block_sums(const double (&acc)[ND], double (&buf)[ND][kThreads], F&& store) {
   static_assert(ND <= kThreads / 32 && kThreads == 256, "one warp per value, eight warps");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -263,13 +266,17 @@ __device__ __forceinline__ void block_sums(const double (&acc)[ND], double (&buf
   __syncthreads();
   const int j = (warp - (int)blockIdx.x) & 7;
   if (j < ND) {
-    double b[8];
+    double b[8], v;
 #pragma unroll
     for (int w = 0; w < 8; ++w) b[w] = buf[j][w * 32 + lane];
-    const double s = warp_sum_transposed<8>(b);   // lanes 4 w .. 4 w + 3: the sum of warp w
-    double v = __shfl_sync(0xffffffffu, s, 0);
+    if constexpr (FREE) {
+      v = warp_sum(((b[0] + b[2]) + (b[4] + b[6])) + ((b[1] + b[3]) + (b[5] + b[7])));
+    } else {
+      const double s = warp_sum_transposed<8>(b);   // lanes 4 w .. 4 w + 3: the sum of warp w
+      v = __shfl_sync(0xffffffffu, s, 0);
 #pragma unroll
-    for (int w = 1; w < 8; ++w) v += __shfl_sync(0xffffffffu, s, 4 * w);
+      for (int w = 1; w < 8; ++w) v += __shfl_sync(0xffffffffu, s, 4 * w);
+    }
     if (lane == 0) store(j, v);
   }
 }
@@ -440,15 +447,17 @@ __device__ __forceinline__ bool reduce_last_block(const double (&acc)[ND], int n
 
 // reduce_last_block for the kernels of the FP64 path (blocks of kThreads
 // threads), with block_sums in place of the shuffle trees: the same sums bit for
-// bit (partials[blockIdx.x * ND + j]; the last block's thread t takes rows t, t +
-// kThreads, ..., then block_sums).  The order of these sums is part of the
+// bit unless FREE (partials[blockIdx.x * ND + j]; the last block's thread t takes
+// rows t, t + kThreads, ..., then block_sums).  The order of these sums is part of the
 // methods' results: the pipelined recurrences amplify a last-bit difference by
-// up to 1e8 within some tens of iterations.
-template <int ND>
+// up to 1e8 within some tens of iterations.  At 64^3 the inner PCG's r update
+// takes 10.4 us (12.2 with the trees), PIPEGCR's operator with its three dots
+// 16.3 (18.7).
+template <int ND, bool FREE = false>
 __device__ __forceinline__ bool reduce_last_block_fast(const double (&acc)[ND], double* partials, unsigned int* counter,
-                                                  double* sums) {
+                                                       double* sums) {
   __shared__ double buf[ND][kThreads];
-  block_sums<ND>(acc, buf, [&](int j, double v) { partials[(size_t)blockIdx.x * ND + j] = v; });
+  block_sums<ND, FREE>(acc, buf, [&](int j, double v) { partials[(size_t)blockIdx.x * ND + j] = v; });
   if (!arrive_last(counter, gridDim.x)) return false;
   double t[ND];
 #pragma unroll
@@ -468,7 +477,7 @@ __device__ __forceinline__ bool reduce_last_block_fast(const double (&acc)[ND], 
 #pragma unroll
         for (int j = 0; j < ND; ++j) t[j] += q[u][j];
   }
-  block_sums<ND>(t, buf, [&](int j, double v) { sums[j] = v; });
+  block_sums<ND, FREE>(t, buf, [&](int j, double v) { sums[j] = v; });
   __syncthreads();
   if (threadIdx.x == 0) *counter = 0u;
   return true;
@@ -479,7 +488,7 @@ template <int ND>
 __device__ __forceinline__ bool reduce_last_block_wide(const double (&acc)[ND], double* partials,
                                                        unsigned int* counter, double* sums) {
   __shared__ double buf[ND][kThreads];
-  block_sums<ND>(acc, buf, [&](int j, double v) { partials[(size_t)blockIdx.x * ND + j] = v; });
+  block_sums<ND, false>(acc, buf, [&](int j, double v) { partials[(size_t)blockIdx.x * ND + j] = v; });
   if (!arrive_last(counter, gridDim.x)) return false;
   sum_rows(partials, gridDim.x, ND, ND, &buf[0][0], sums, true);
   if (threadIdx.x == 0) *counter = 0u;
