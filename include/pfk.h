@@ -505,9 +505,10 @@ pfk_status pfk_probe_fp64_fma(pfk_context* ctx, int iters, double* tflops, doubl
 /* Largest operator size accepted by pfk_pc_apply_inner_pcg_noalloc. */
 #define PFK_NOALLOC_MAX_N 262144
 
-/* y = B(v) for the FP64 inner Jacobi-PCG preconditioner (the same result as
+/* y = B(v) for the FP64 inner Jacobi-PCG preconditioner (the result of
  * pfk_pc_apply with a PFK_PC_INNER_PCG / PFK_FP64 preconditioner of
- * `inner_iters` iterations on `op`), without allocating any device memory.
+ * `inner_iters` iterations on `op`, up to the rounding of the inner products,
+ * which are added in another order), without allocating any device memory.
  * The paper has no counterpart: this is a library service for callers that
  * cannot allocate device memory at the point where they apply the
  * preconditioner -- for instance a framework that has handed all device memory

@@ -1,11 +1,11 @@
 // FP64 inner Jacobi-PCG (Alg. 3, M^-1 = D^-1) in one cooperative launch, for
 // grids whose inner vectors fit in the SMs' shared memory.
 //
-// As separate kernels (pc.cu) an application of k inner iterations is 3k + 1
+// As separate kernels (pc.cu) an application of k inner iterations is 3k
 // launches.  Below about a million cells each of them spends most of its time
 // outside its loop: launch and block ramp-up, the L2 round trips of its control
-// words, the shuffle trees and the last-block combine (64^3: 14 kernels of 4.6
-// to 8.8 us for 27 us of FP64 work).  Here every SM keeps one block with a
+// words, the sums and the last-block combine (64^3: 12 kernels of 4 to 15 us for
+// 27 us of FP64 work).  Here every SM keeps one block with a
 // fixed range of consecutive cells; r, s (D^-1 r after the r update), x and p of
 // those cells stay in shared memory for the whole application, p also in global
 // memory for the stencils of the neighbouring blocks, and the blocks meet at a
@@ -13,7 +13,10 @@
 // iteration (<s, p>, <D^-1 r, r>, p complete).  A reduction writes one partial
 // sum per block before its barrier; after it every block adds all partial sums
 // in the same order, so all hold bitwise the same scalars.  The statements per
-// cell are those of the separate kernels.
+// cell are those of the separate kernels; the sums are added in another order,
+// so single applications and the blocking methods (FCG, GCR, FGMRES) use this
+// form and the pipelined methods, which amplify that difference, do not
+// (PcCall::pinned).
 //
 // A barrier and the sum behind it take 3 to 4 us, in which the warps that do
 // not wait have nothing to do, so work that depends on neither is placed there:
@@ -22,8 +25,8 @@
 // 88 -> 85 us; 101 x 97 x 93: 146 -> 140 us).  The registers are kept to two
 // blocks per SM although a launch has one, so that the applications of two
 // solves on different streams run side by side: with all registers for one
-// block 64^3 takes 83 us, but a burst of small solves on several workers 29 ms
-// instead of 21.
+// block 64^3 takes 83 us, but a burst of eight small solves on four workers, all
+// with this form, 29 ms instead of 21.
 //
 // Every wait is bounded (pfk_solve_params' barrier_timeout_us, else 2 s): a wait
 // that runs out raises an abort word that ends all other waits, the blocks that

@@ -87,7 +87,8 @@ class Method {
 // body(e, v_e) adds the caller's own products.  The loop is instantiated for
 // window sizes rounded up to 4: with one loop for 32 slots the guarded products
 // of the empty slots were issued all the same (101x97x93: 79 us at every window
-// size).  The order of a thread's sum depends on the grid alone.
+// size; PIPEGCR at 64^3: 45 us at the median window and 63 at the largest, now 35
+// and 43).  The order of a thread's sum depends on the grid alone.
 constexpr int kWinThreads = 128;
 constexpr int kWinBlocksPerSm = 4;   // base methods: 128 registers
 
