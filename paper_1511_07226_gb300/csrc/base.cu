@@ -436,7 +436,7 @@ static cudaError_t launch_apply_dots(const SolveEnv& env, double* P, double* S, 
     const bool adv = op->adv[0] != 0.0 || op->adv[1] != 0.0 || op->adv[2] != 0.0;
     const int slots = kWalkBlocksPerSm * env.ctx->num_sms;
     const int units = tiled_stencil_setup<double, double>(T, op, op->d, op->kx, op->ky, op->kz, slots);
-    const int64_t cap = env.partials_cap / ND;
+    const int64_t cap = env.partials_cap / 5;   // (part of the order: blocks take units u, u + blocks, ...)
     const int blocks = (int)(units < cap ? units : cap);
     if (adv) base_apply_dots_walk<true, MODE><<<blocks, kTileThreads, 0, env.st>>>(T, P, S, r, env.N, env.ctl, env.partials);
     else base_apply_dots_walk<false, MODE><<<blocks, kTileThreads, 0, env.st>>>(T, P, S, r, env.N, env.ctl, env.partials);

@@ -70,6 +70,8 @@ CASES = {
     "prec_gcr_csr": _c("prec", "gcr", (300, 210, 1), 30, 16, precision="fp32", storage="csr"),
     "prec_fgmres": _c("prec", "fgmres", (118, 112, 127), 25, 25, pc="chebyshev", inner=8, vel=ADV, precision="bf16"),
     "prec_fgmres_8": _c("prec", "fgmres", (40, 33, 21), 7, 14, precision="fp32"),
+    "prec_fcg_units": _c("prec", "fcg", (2048, 1500, 1), 8, 8, precision="fp32"),   # more work units than blocks
+    "prec_gcr_units": _c("prec", "gcr", (1500, 2048, 2), 4, 6, pc="chebyshev", precision="bf16"),
     "prec_fgmres_32": _c("prec", "fgmres", (40, 33, 21), 32, 32, pc="chebyshev", vel=ADV, precision="fp32"),
 }
 
